@@ -66,7 +66,6 @@ struct pico_ctx {
   int64_t nsamp = 0;
   float2* Gt = nullptr;  // Toeplitz / 2-D intermediates [B][nc][n][L]
   bool mask2d = false;   // Cartesian with a 2-D sampling mask (normal operator by the 2-D passes, L = n)
-  int toep_rl = 16;      // image rows per block of the Toeplitz / 2-D row passes
   // nonlinear CS state (pico_cs_*)
   bool cs_ready = false;
   int cs_iters = 0, cs_levels = 0;
@@ -318,7 +317,8 @@ void op_apply(pico_ctx* c, const float2* x, float2* y, int nb, float lam) {
     pico::launch_cart_apply(c->cop, x, y, nb, lam, c->stream);
   } else {
     Launch L(c, 0, 3);
-    pico::launch_toep_apply(c->sop, x, y, c->Gt, nb, lam, c->stream);
+    if (!pico::launch_toep_apply(c->sop, x, y, c->Gt, nb, lam, c->stream))
+      c->host_fail = "normal operator launch failed (tensor map encoding)";
   }
 }
 
@@ -355,7 +355,8 @@ void op_cg_normal(pico_ctx* c, int nb, int it, float lam) {
     pico::launch_cart_cg_normal(c->cop, c->cg, nb, it, lam, c->stream);
   } else {
     Launch L(c, 0, 3);
-    pico::launch_toep_cg_normal(c->sop, c->cg, c->Gt, nb, it, lam, c->stream);
+    if (!pico::launch_toep_cg_normal(c->sop, c->cg, c->Gt, nb, it, lam, c->stream))
+      c->host_fail = "normal operator launch failed (tensor map encoding)";
   }
 }
 
@@ -653,7 +654,6 @@ pico_status cart2d_setup(pico_ctx* c, const pico_operator_desc* d, int img, int 
   c->sop.tw2 = c->tw2;
   c->sop.That = c->That;
   c->sop.err = c->g_err;
-  c->sop.row_lines = c->toep_rl;
   c->twx = c->tw2;
   c->tw = c->tw2;
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return cuda_check(c, "2-D mask set-up");
@@ -759,8 +759,7 @@ pico_status spiral_setup(pico_ctx* c, const pico_operator_desc* d, int img, int 
 
   c->sop = pico::SpiralOp{img,      L,         nc,         P1,          P2,           c->smaps,
                           c->tw2,   c->That,   c->deapod,  M,           c->u,         c->cphase,
-                          c->tile_ptr, c->tile_idx, (float)beta, (float)hw, (float)(1.0 / i0b), c->g_err,
-                          c->toep_rl};
+                          c->tile_ptr, c->tile_idx, (float)beta, (float)hw, (float)(1.0 / i0b), c->g_err};
   // the Kaiser-Bessel window of every sample, once (the gridding of each PMR
   // replica batch and pico_adjoint look the weights up)
   if ((st = dalloc(c, &c->grid_w, std::max<size_t>(1, pico::grid_table_floats(M)))) != PICO_OK) return st;
@@ -900,15 +899,6 @@ bool want_onchip(const pico_operator_desc* d) {
   if (e && std::string(e) == "fft") return false;
   return pico::colcg_small_supported(d->ny);
 }
-// Image rows per block of the Toeplitz / 2-D-mask row passes: 4 (blocks of
-// a quarter of the threads, four per SM) unless PICO_TOEP_ROWS=16 in the
-// environment asks for one block of 16 rows per SM.  The p^H q partials per
-// image are one per row block.
-int toep_row_lines() {
-  const char* e = std::getenv("PICO_TOEP_ROWS");
-  return e && std::atoi(e) == 16 ? 16 : 4;
-}
-
 size_t onchip_extra_bytes(const pico_operator_desc* d, int64_t B) {
   return (size_t)d->nx * d->ny * d->ny * 8 + 4 + (size_t)d->ny * 16 + (size_t)B * d->nx * (8 + 8 + 4 + 16 + 16);
 }
@@ -1060,8 +1050,7 @@ pico_status init_impl(const pico_operator_desc* d, void* cuda_stream, size_t hbm
     if (c->ny != c->nx) return fail(c, PICO_E_UNSUPPORTED, "2-D masks need square images");
     if (!pico::grid_split(img, &P1, &P2) || !pico::fft_length_supported(img))
       return fail(c, PICO_E_UNSUPPORTED, "image size has no 2-D FFT split in this build");
-    c->toep_rl = toep_row_lines();
-    PA = (img + c->toep_rl - 1) / c->toep_rl;
+    PA = img / pico::kRowLines;
     extra = std::max((size_t)B * nc * n, (size_t)n) * 8 + (size_t)n * 5 + (size_t)img * 8;
   } else if (c->kind == PICO_CARTESIAN) {
     if (!pico::cart_supported(c->ny, c->nx, &N1, &N2, &M1, &M2))
@@ -1081,8 +1070,7 @@ pico_status init_impl(const pico_operator_desc* d, void* cuda_stream, size_t hbm
     if (kbw < 2 || kbw > 8 || (kbw & 1)) return fail(c, PICO_E_UNSUPPORTED, "kb_width must be 2, 4, 6 or 8");
     if (!pico::spiral_supported(img, &P1, &P2))
       return fail(c, PICO_E_UNSUPPORTED, "spiral image size has no 2N grid split in this build");
-    c->toep_rl = toep_row_lines();
-    PA = (img + c->toep_rl - 1) / c->toep_rl;
+    PA = img / pico::kRowLines;
     c->nsamp = d->nsamp;
     extra = std::max((size_t)B * nc * img * L, (size_t)L * L) * 8 + (size_t)L * L * 4 + (size_t)img * 4 + (size_t)L * 8 +
             (size_t)c->nsamp * (8 + 8 + 8 + 16 + 88) + (size_t)(L / 16) * (L / 16) * 4 + 64;
@@ -1225,7 +1213,7 @@ size_t footprint_bytes(const pico_operator_desc* d, bool with_kbuf) {
   const int64_t PB = (n + kVecPerBlock - 1) / kVecPerBlock;
   int64_t PA, extra, kbuf;
   if (d->kind == PICO_CARTESIAN && d->mask_2d) {
-    PA = (d->ny + toep_row_lines() - 1) / toep_row_lines();
+    PA = d->ny / kRowLines;
     extra = std::max(B * nc * n, n) * 8 + n * 5 + (int64_t)d->ny * 8;
     kbuf = B * nc * n * 8;
   } else if (d->kind == PICO_CARTESIAN) {
@@ -1239,7 +1227,7 @@ size_t footprint_bytes(const pico_operator_desc* d, bool with_kbuf) {
     }
   } else {
     const int64_t img = d->ny, L = 2 * img;
-    PA = (img + toep_row_lines() - 1) / toep_row_lines();
+    PA = img / kRowLines;
     extra = std::max(B * nc * img * L, L * L) * 8 + L * L * 4 + img * 4 + L * 8 + d->nsamp * (56 + 88) +
             (L / 16) * (L / 16) * 4 + 64;
     kbuf = B * nc * 4 * n * 8;

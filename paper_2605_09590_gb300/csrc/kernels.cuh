@@ -233,20 +233,26 @@ struct SpiralOp {
   const int* tile_idx;      // samples touching each tile (with the kernel half-width)
   float beta, halfw, inv_i0beta;
   int* err;                 // first failure code of a bounded wait (device), or nullptr
-  int row_lines;            // image rows per block of the Toeplitz row passes: 4 or 16 (0 = 16)
   const float* gw;          // [M][2][kMaxTaps] Kaiser-Bessel weights of each sample's window (x, then y)
   const int2* go;           // [M] wrapped first grid index (x, y) of each sample's window
 };
+// Image rows per block of the Toeplitz / 2-D-mask row passes (every supported
+// image side is a multiple); one p^H q partial per row block.
+constexpr int kRowLines = 4;
 // 3-D tensor map over `planes` planes of rows x L complex64 values (8-byte
 // elements), boxes of `cols` x `box_rows` values (the column pass's staging)
 bool encode_plane_map(CUtensorMap* m, const void* base, int rows, int L, int64_t planes, int cols, int box_rows);
+// 3-D tensor map over grid rows of P1 x P2 complex64 values, boxes of box_rows
+// rows swizzled by their P2 values (the inverse row pass's exchange layout)
+bool encode_row_map(CUtensorMap* m, const void* base, int P1, int P2, int64_t rows, int box_rows);
 bool spiral_supported(int n, int* P1, int* P2);
 bool grid_split(int L, int* P1, int* P2);  // split of a 2-D pass length (Toeplitz or 2-D Cartesian)
 void launch_toep_h(const float* traj, int64_t M, int n, float2* c, cudaStream_t s);
 void launch_toep_fft2(const SpiralOp& op, float2* c, cudaStream_t s);  // c <- DFT_2D(c)
 void launch_toep_finalize(const float2* c, int L, float scale, float* That, cudaStream_t s);
-void launch_toep_apply(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam, cudaStream_t s);
-void launch_toep_cg_normal(const SpiralOp& op, const CgArgs& a, float2* G, int nb, int it, float lam,
+// The normal operator in three passes; false (nothing usable written) if a tensor map cannot be encoded
+bool launch_toep_apply(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam, cudaStream_t s);
+bool launch_toep_cg_normal(const SpiralOp& op, const CgArgs& a, float2* G, int nb, int it, float lam,
                            cudaStream_t s);
 // the per-sample gridding windows (set-up; gw holds grid_table_floats(M) floats)
 size_t grid_table_floats(int64_t M);

@@ -7,7 +7,7 @@
 namespace pico {
 
 template <int P1, int P2>
-void launch_toep_normal_t(const SpiralOp&, const float2*, float2*, float2*, int, float, const CgArgs*, int,
+bool launch_toep_normal_t(const SpiralOp&, const float2*, float2*, float2*, int, float, const CgArgs*, int,
                           cudaStream_t);
 template <int P1, int P2>
 void launch_fft2_t(float2*, const float2*, int, int, bool, cudaStream_t);
@@ -251,19 +251,21 @@ void launch_toep_finalize(const float2* c, int L, float scale, float* T, cudaStr
   k_toep_finalize<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(c, cnt, scale, T);
 }
 
-void launch_toep_apply(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam, cudaStream_t s) {
+bool launch_toep_apply(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam, cudaStream_t s) {
 #define PICO_CASE(LL, A, B) \
   if (op.P1 == A && op.P2 == B) return launch_toep_normal_t<A, B>(op, x, y, G, nb, lam, nullptr, 0, s);
   PICO_GRID_SIZES(PICO_CASE)
 #undef PICO_CASE
+  return false;
 }
 
-void launch_toep_cg_normal(const SpiralOp& op, const CgArgs& a, float2* G, int nb, int it, float lam,
+bool launch_toep_cg_normal(const SpiralOp& op, const CgArgs& a, float2* G, int nb, int it, float lam,
                            cudaStream_t s) {
 #define PICO_CASE(LL, A, B) \
   if (op.P1 == A && op.P2 == B) return launch_toep_normal_t<A, B>(op, nullptr, nullptr, G, nb, lam, &a, it, s);
   PICO_GRID_SIZES(PICO_CASE)
 #undef PICO_CASE
+  return false;
 }
 
 size_t grid_table_floats(int64_t M) { return (size_t)M * 2 * kMaxTaps; }

@@ -27,6 +27,7 @@
 
 namespace pico {
 
+
 __device__ __forceinline__ const double* sp_rr(const CgArgs& a, int b, int it) {
   return a.rr_part + ((size_t)b * (a.itmax + 1) + it) * a.PB;
 }
@@ -47,14 +48,54 @@ __device__ __forceinline__ void cg_scalars(const CgArgs& a, int b, int it, int* 
   }
 }
 
-// Row-pass blocks of RL image rows: RL = 16 (one block of up to 480 threads
-// per SM) or RL = 4 (a quarter of the threads, four blocks per SM, so that
-// the blocks' global loads and stores overlap one another's transforms).
-template <int P1, int P2, int RL>
-struct RowSplit {
-  static constexpr int NT = (RL * (P1 > P2 ? P1 : P2) + 31) / 32 * 32;
-  static constexpr int MINB = RL <= 4 ? 4 : RL <= 8 ? 2 : 1;
-  static constexpr size_t buf = (size_t)RL * P2 * Split<P1, P2>::LD * sizeof(float2);
+// Row passes.  A block owns kRowLines image rows of one image and walks the
+// coils in steps of CS at once, so that the b-jobs (one per coil, row and
+// frequency group k2) fill all NT threads; the a-jobs (one per row and n1) of
+// GA coil subgroups fill up to NT threads too, each thread working through
+// CA = CS / GA coils of a step.  kRowLines divides every supported side.
+//
+// Before, a block's one coil at a time left half of its threads without a b-job,
+// the strided twiddle look-ups made up most of the shared-memory wavefronts, and
+// every coil waited for its own global loads (ncu: issue 30-36 %, barrier and
+// load stalls 6 of 8 warps): 32 images at L = 480, forward 176 -> 132 us,
+// inverse 221 -> 157 us, now at 55 % of the DRAM rate.
+//
+// Exchange layout: a line of each (coil, image row) holds P1 rows of P2 values,
+// row n1 the P2 values of that n1, with the 16-byte chunk of value k at
+// (k >> 1) ^ (n1 & 7) (64-byte rows: ^ ((n1 >> 1) & 3)) -- the TMA swizzle of
+// that row width, lines padded to the pattern's period.  a-jobs (consecutive
+// lanes, consecutive n1) move two values per 16-byte access, b-jobs
+// (consecutive lanes, consecutive k2) one value per 8-byte access, both without
+// bank conflicts, and the inverse pass's rows arrive in it directly.  The
+// twiddles of the a-jobs are stored [k][n1] for the same reason: the strided
+// look-ups W^(n1 k) of the plain table cost more shared-memory wavefronts than
+// the data.
+
+template <int P1, int P2, int NT_>
+struct RowPass {
+  static constexpr int RL = kRowLines;
+  static constexpr int NT = NT_;
+  static constexpr int CS = NT / (RL * P2);          // coils per step
+  static constexpr int ga(int nin) {
+    int g = CS;
+    while (RL * P1 * g > NT || g > nin) g /= 2;
+    return g;
+  }
+  static constexpr int GA = ga(P2 / 2);               // coil subgroups of the a-jobs
+  static constexpr int CA = CS / GA;                  // coils per a-thread and step
+  static constexpr int AT = RL * P1 * GA;             // a-threads
+  static constexpr int RB = P2 * 8;                   // bytes of an exchange row
+  static constexpr int period = P2 == 16 ? 1024 : 512;  // of the swizzle pattern
+  static constexpr int line = (P1 * RB + period - 1) / period * period;  // bytes of a line
+  static constexpr size_t slot = (size_t)RL * line;
+  static constexpr size_t tw = (size_t)P1 * P2 * sizeof(float2);
+  // exchange slots, sensitivity rows, twiddles, two mbarriers, alignment slack
+  static constexpr size_t smem(int n) { return 1024 + CS * slot + (size_t)CS * RL * n * 8 + tw + 16; }
+  // byte offset of value k of row n1 in a line (the XOR is on bits 4 ..)
+  static __device__ __forceinline__ uint32_t at(int n1, int k) {
+    const uint32_t sw = P2 == 16 ? (n1 & 7) : ((n1 >> 1) & 3);
+    return (uint32_t)(n1 * RB) + ((((uint32_t)(k >> 1) ^ sw) << 4) | ((k & 1) << 3));
+  }
 };
 
 // ---------------------------------------------------------------------------
@@ -62,171 +103,187 @@ struct RowSplit {
 // ---------------------------------------------------------------------------
 // PAD: the grid is 2N (Toeplitz embedding, image in the first half of each
 // line); otherwise L = N (2-D Cartesian masks: plain 2-D DFT, no padding).
-template <int P1, int P2, bool CG, bool PAD, int RL>
-__global__ void __launch_bounds__(RowSplit<P1, P2, RL>::NT, RowSplit<P1, P2, RL>::MINB)
+// The next step's sensitivity rows (contiguous) arrive by bulk copies while the
+// b-jobs of the current step run.
+template <int P1, int P2, bool CG, bool PAD, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT)
     k_toep_rows_fwd(SpiralOp op, const float2* __restrict__ xin, float2* __restrict__ G, CgArgs a, int it) {
+  using Rp = RowPass<P1, P2, NT>;
+  constexpr int RL = Rp::RL, CS = Rp::CS, GA = Rp::GA, CA = Rp::CA;
   constexpr int NIN = PAD ? P2 / 2 : P2;  // samples n1 + P1 n2 inside the image: n2 < NIN
   constexpr int L = P1 * P2;
-  constexpr int NT = RowSplit<P1, P2, RL>::NT;
+  constexpr int N = PAD ? L / 2 : L;
   extern __shared__ __align__(16) unsigned char smraw[];
-  float2* buf = reinterpret_cast<float2*>(smraw);
-  float2* tws = buf + RL * P2 * Split<P1, P2>::LD;
+  unsigned char* ex = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
+  float2* sst = reinterpret_cast<float2*>(ex + CS * Rp::slot);  // [CS][RL][N]
+  float2* twt = sst + CS * RL * N;                              // [P2][P1]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(twt + L);
   __shared__ float sh_beta;
   __shared__ int sh_done;
-  const int t = threadIdx.x, b = blockIdx.y, N = op.n;
-  for (int i = t; i < L; i += NT) tws[i] = op.tw2[i];
+  const int t = threadIdx.x, b = blockIdx.y, y0 = blockIdx.x * RL;
+  if (t == 0) {
+    tc::mbar_init(bar, 1);
+    tc::fence_mbar_init();
+  }
+  for (int i = t; i < L; i += NT) twt[i] = op.tw2[(i / P1) * (i % P1)];
   if (CG) cg_scalars(a, b, it, &sh_done, &sh_beta);
   __syncthreads();
   if (CG && blockIdx.x == 0 && t == 0 && a.done) a.done[b] = sh_done;  // for the column pass
   if (CG && sh_done) return;
+  auto issue = [&](int c0) {  // sensitivity rows of a step
+    const int cn = min(CS, op.nc - c0);
+    tc::mbar_expect_tx(bar, (uint32_t)(cn * RL * N * 8));
+    for (int c = 0; c < cn; ++c)
+      tc::bulk_load(sst + c * RL * N, op.smaps + ((size_t)(c0 + c) * N + y0) * N, RL * N * 8, bar);
+  };
+  if (t == 0) issue(0);
 
-  const int ra = t / P1, n1 = t % P1;
-  const bool ajob = t < RL * P1;
-  const int ya = blockIdx.x * RL + ra;
-  const bool aval = ajob && ya < N;
-  const int rb = t / P2, k2 = t % P2;
-  const bool bjob = t < RL * P2;
-  const int yb = blockIdx.x * RL + rb;
-  const bool bval = bjob && yb < N;
-  const size_t img = (size_t)b * N * N;
-
-  float2 p[P2];
+  const int g = t / (RL * P1), mm = t - g * (RL * P1), ra = mm / P1, n1 = mm - ra * P1;
+  const bool ajob = t < Rp::AT;
+  const int cb = t / (RL * P2), rb = (t / P2) % RL, k2 = t % P2;
+  float2 p[NIN];
   if (ajob) {
     const float beta = CG ? sh_beta : 0.f;
+    const size_t row = ((size_t)b * N + y0 + ra) * N + n1;
 #pragma unroll
-    for (int n2 = 0; n2 < P2; ++n2) {
-      const int x = n1 + P1 * n2;
-      float2 v = make_float2(0.f, 0.f);
-      if (aval && n2 < NIN) {
-        const size_t idx = img + (size_t)ya * N + x;
-        if (CG) {
-          const float2 r = a.R[idx];
-          if (it > 0) {
-            const float2 po = a.P[idx];
-            v = make_float2(fmaf(beta, po.x, r.x), fmaf(beta, po.y, r.y));
-          } else {
-            v = r;
+    for (int n2 = 0; n2 < NIN; ++n2) {
+      const size_t idx = row + P1 * n2;
+      if (CG) {
+        float2 v = a.R[idx];
+        if (it > 0) {
+          const float2 po = a.P[idx];
+          v = make_float2(fmaf(beta, po.x, v.x), fmaf(beta, po.y, v.y));
+        }
+        p[n2] = v;
+      } else {
+        p[n2] = xin[idx];
+      }
+    }
+    if (CG && GA == 1)
+#pragma unroll
+      for (int n2 = 0; n2 < NIN; ++n2) a.P[row + P1 * n2] = p[n2];
+  }
+  if (CG && GA > 1) {  // every subgroup has read the old direction before one writes the new
+    __syncthreads();
+    if (t < RL * P1)
+#pragma unroll
+      for (int n2 = 0; n2 < NIN; ++n2) a.P[((size_t)b * N + y0 + ra) * N + n1 + P1 * n2] = p[n2];
+  }
+  bool ok = true;
+  int phase = 0;
+  for (int c0 = 0; c0 < op.nc; c0 += CS, phase ^= 1) {
+    if (ok && !tc::mbar_wait(bar, phase)) {  // reported by pico_sync; the block runs on so that its barriers pair up
+      ok = false;
+      if (op.err) atomicCAS(op.err, 0, 11);
+    }
+    if (ajob) {
+#pragma unroll
+      for (int j = 0; j < CA; ++j) {
+        const int cs = j * GA + g;
+        if (c0 + cs < op.nc) {
+          float2 z[P2];
+          const float2* S = sst + (cs * RL + ra) * N + n1;
+#pragma unroll
+          for (int n2 = 0; n2 < P2; ++n2) z[n2] = n2 < NIN ? cmul(S[P1 * n2], p[n2]) : make_float2(0.f, 0.f);
+          dft_nz<P2, -1, NIN>(z);
+          unsigned char* e = ex + cs * Rp::slot + ra * Rp::line;
+#pragma unroll
+          for (int k = 0; k < P2; k += 2) {
+            const float2 u = k == 0 ? z[0] : cmul(z[k], twt[k * P1 + n1]), v = cmul(z[k + 1], twt[(k + 1) * P1 + n1]);
+            *reinterpret_cast<float4*>(e + Rp::at(n1, k)) = make_float4(u.x, u.y, v.x, v.y);
           }
-          a.P[idx] = v;
-        } else {
-          v = xin[idx];
         }
       }
-      p[n2] = v;
     }
-  }
-  for (int c = 0; c < op.nc; ++c) {
-    if (ajob) {
-      float2 z[P2];
-      const float2* __restrict__ S = op.smaps + ((size_t)c * N + (aval ? ya : 0)) * N;
-#pragma unroll
-      for (int n2 = 0; n2 < P2; ++n2) {
-        const int x = n1 + P1 * n2;
-        z[n2] = (aval && n2 < NIN) ? cmul(__ldg(S + x), p[n2]) : make_float2(0.f, 0.f);
-      }
-      rowa_store<P1, P2, -1, NIN>(z, n1, ra, buf, tws);
-    }
-    __syncthreads();
-    if (bval) {
+    __syncthreads();  // exchange slots full, sensitivities read
+    if (t == 0 && c0 + CS < op.nc) issue(c0 + CS);
+    if (c0 + cb < op.nc) {
       float2 y[P1];
-      rowb_load<P1, P2, -1>(y, k2, rb, buf);
-      float2* __restrict__ g = G + (((size_t)b * op.nc + c) * N + yb) * L;
+      const unsigned char* e = ex + cb * Rp::slot + rb * Rp::line;
 #pragma unroll
-      for (int k1 = 0; k1 < P1; ++k1) g[k2 + P2 * k1] = y[k1];
+      for (int m = 0; m < P1; ++m) y[m] = *reinterpret_cast<const float2*>(e + Rp::at(m, k2));
+      DFT<P1, -1>::run(y);
+      float2* __restrict__ gr = G + (((size_t)b * op.nc + c0 + cb) * N + y0 + rb) * L + k2;
+#pragma unroll
+      for (int k1 = 0; k1 < P1; ++k1) gr[P2 * k1] = y[k1];
     }
-    __syncthreads();
+    __syncthreads();  // the slots are rewritten by the next step
   }
 }
 
 // ---------------------------------------------------------------------------
 // Pass 2: columns of the grid: FFT (rows >= N zero), x T^, inverse FFT, rows < N
 // ---------------------------------------------------------------------------
+// Persistent: each block walks work items (plane, group of CL grid columns) and
+// one thread brings the next item's N x CL input values into a staging buffer
+// with TMA tensor loads while the block transforms the current item, so the
+// global-load latency of a plane does not stall every thread at its start.
 // done: per-image stop flags of the CG iteration (nullptr outside CG); planes of
-// converged images are skipped
+// converged images are skipped.
+//
+// CL = 16 columns: a half-warp's 16 columns fill a 128-byte shared-memory
+// wavefront and a full 128-byte line of the grid, and blocks of P2 x 16 threads
+// (one b-job each) run two or three to an SM, so one block's barriers and loads
+// overlap another's arithmetic.  96 images, 240 x 240, 20 coils (L = 480), whole
+// normal operator: groups of 30 columns (one 480-thread block per SM) 2397 us,
+// 16 columns 2287 us, 8 columns 2403 us (64-byte global accesses), 4 columns
+// 2824 us.  The twiddles are read two at a time, [n1][k] with padded rows, by
+// the a-jobs in both directions (single look-ups W^(n1 k) by a- and b-jobs:
+// 2084 us against 2045 us, with the row passes below in place).
+// Bound by shared-memory wavefronts and the FP32 pipes at about half each (ncu,
+// 32 images: 56 % and 50 %): every value crosses shared memory five times, and
+// two blocks of 8 warps overlap the two pipes only partly.
+template <int P1, int P2>
+struct ColsW {
+  static constexpr int CL = 16;                    // grid columns per item
+  static constexpr int NT = P2 * CL;               // one b-job per thread
+  static constexpr int KS = P1 * CL;               // k2 stride of the exchange buffer
+  static constexpr int TS = P2 + 2;                // twiddle row, padded against bank conflicts
+  static constexpr size_t smem(int n) {
+    return 1024 + ((size_t)n * CL + (size_t)P2 * KS + P1 * TS) * sizeof(float2) + 16;
+  }
+  // blocks per SM to compile for: three of 256 threads (six of 128) where the
+  // shorter DFT and the shared memory allow, otherwise two (four)
+  static constexpr int blocks(int n) {
+    const int want = (P1 <= 20 ? 768 : 512) / NT, fit = (int)((size_t)227 * 1024 / (smem(n) + 1024));
+    return fit < 1 ? 1 : fit < want ? fit : want;
+  }
+};
 template <int P1, int P2, bool PAD>
-__global__ void __launch_bounds__(Split<P1, P2>::NT, 1)
-    k_toep_cols(SpiralOp op, float2* __restrict__ G, const int* __restrict__ done) {
-  constexpr int NIN = PAD ? P2 / 2 : P2;
-  constexpr int L = P1 * P2;
-  constexpr int NT = Split<P1, P2>::NT;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  float2* buf = reinterpret_cast<float2*>(smraw);
-  float2* tws = buf + L * kLines;
-  const int t = threadIdx.x, N = op.n;
-  if (done && done[blockIdx.y / op.nc]) return;
-  for (int i = t; i < L; i += NT) tws[i] = op.tw2[i];
-  __syncthreads();
-  const int ln = t % kLines, job = t / kLines;
-  const int kx = blockIdx.x * kLines + ln;  // grid column (always < L: L is a multiple of 16)
-  float2* __restrict__ g = G + (size_t)blockIdx.y * N * L;  // (b, c) plane [N][L]
-  const int n1 = job, k2 = job;
-  if (job < P1) {
-    float2 z[P2];
-#pragma unroll
-    for (int n2 = 0; n2 < P2; ++n2) {
-      const int y = n1 + P1 * n2;  // rows >= N (n2 >= NIN) are the zero padding
-      z[n2] = n2 < NIN ? g[(size_t)y * L + kx] : make_float2(0.f, 0.f);
-    }
-    cola_store<P1, P2, -1, NIN>(z, n1, ln, buf, tws);
-  }
-  __syncthreads();
-  if (job < P2) {
-    float2 y[P1];
-    colb_load<P1, P2>(y, k2, ln, buf);
-    DFT<P1, -1>::run(y);
-#pragma unroll
-    for (int k1 = 0; k1 < P1; ++k1) y[k1] = cscale(y[k1], __ldg(op.That + (size_t)(k2 + P2 * k1) * L + kx));
-    colb_inv_store<P1, P2>(y, k2, ln, buf, tws);
-  }
-  __syncthreads();
-  if (job < P1) {
-    float2 z[P2];
-    cola_load<P1, P2, 1>(z, n1, ln, buf);
-#pragma unroll
-    for (int n2 = 0; n2 < NIN; ++n2) g[(size_t)(n1 + P1 * n2) * L + kx] = z[n2];  // rows < N only
-  }
-}
-
-// The same pass for splits with P1 > P2, persistent: each block walks work
-// items (plane, group of P1 grid columns) and one thread brings the next
-// item's N x P1 input values into a staging buffer with TMA tensor loads
-// while the block transforms the current item, so the global-load latency of
-// a plane no longer stalls every thread at its start.  With P1 columns per
-// item the b-jobs (the heavy DFT_P1 pair and the T^ product) occupy all
-// P2 x P1 threads; the light DFT_P2 a-jobs take P1 / P2 rounds.
-template <int P1, int P2, bool PAD>
-__global__ void __launch_bounds__(P1 * P2, (P1 * P2 <= 320 ? 2 : 1))
+__global__ void __launch_bounds__(ColsW<P1, P2>::NT, (ColsW<P1, P2>::blocks(PAD ? P1 * P2 / 2 : P1 * P2)))
     k_toep_cols_w(SpiralOp op, const __grid_constant__ CUtensorMap mG, float2* __restrict__ G,
                   const int* __restrict__ done, int nplanes, int box_rows) {
   constexpr int NIN = PAD ? P2 / 2 : P2;
   constexpr int L = P1 * P2;
-  constexpr int NT = L;
-  constexpr int CL = P1;  // grid columns per item
+  constexpr int NT = ColsW<P1, P2>::NT;
+  constexpr int CL = ColsW<P1, P2>::CL;
+  constexpr int NG = L / CL;
+  constexpr int KS = ColsW<P1, P2>::KS, TS = ColsW<P1, P2>::TS;
   extern __shared__ __align__(16) unsigned char smraw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
   const int t = threadIdx.x, N = op.n;          // N input rows per plane
   float2* stage = reinterpret_cast<float2*>(sm);  // [N][CL] input rows of the item
   float2* buf = stage + (size_t)N * CL;           // [k2][n1][CL]
-  float2* tws = buf + (size_t)L * CL;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(tws + L);
+  float2* tws = buf + (size_t)P2 * KS;            // [n1][k]: W^(n1 k)
+  uint64_t* bar = reinterpret_cast<uint64_t*>(tws + P1 * TS);
   int* arrived = reinterpret_cast<int*>(bar + 1);
-  const int items = P2 * nplanes;
+  const int items = NG * nplanes;
   const uint32_t bytes = (uint32_t)N * CL * sizeof(float2);
   if (t == 0) {
     tc::mbar_init(bar, 1);
     tc::fence_mbar_init();
   }
-  for (int i = t; i < L; i += NT) tws[i] = op.tw2[i];
+  for (int i = t; i < L; i += NT) tws[(i / P2) * TS + i % P2] = op.tw2[(i / P2) * (i % P2)];
   __syncthreads();
   auto issue = [&](int w) {
-    const int plane = w / P2, cg = w - plane * P2;
+    const int plane = w / NG, cg = w - plane * NG;
     tc::mbar_expect_tx(bar, bytes);
     for (int r0 = 0; r0 < N; r0 += box_rows) tc::tma_load_3d(stage + (size_t)r0 * CL, &mG, bar, cg * CL, r0, plane);
   };
   if (t == 0 && (int)blockIdx.x < items) issue(blockIdx.x);
   int phase = 0;
   for (int w = blockIdx.x; w < items; w += gridDim.x, phase ^= 1) {
-    const int plane = w / P2, cg = w - plane * P2, x0 = cg * CL;
+    const int plane = w / NG, cg = w - plane * NG, x0 = cg * CL;
     // One thread decides whether the item's copy arrived and the block
     // follows that decision together.  On a timeout it records the error,
     // waits once more (bounded) for the copy still in flight into this
@@ -249,7 +306,13 @@ __global__ void __launch_bounds__(P1 * P2, (P1 * P2 <= 320 ? 2 : 1))
         float2 z[P2];
 #pragma unroll
         for (int n2 = 0; n2 < P2; ++n2) z[n2] = n2 < NIN ? stage[(n1 + P1 * n2) * CL + ln] : make_float2(0.f, 0.f);
-        cola_store<P1, P2, -1, NIN, CL>(z, n1, ln, buf, tws);
+        dft_nz<P2, -1, NIN>(z);
+#pragma unroll
+        for (int k = 0; k < P2; k += 2) {
+          const float4 w = *reinterpret_cast<const float4*>(tws + n1 * TS + k);
+          buf[k * KS + n1 * CL + ln] = k == 0 ? z[0] : cmul(z[k], make_float2(w.x, w.y));
+          buf[(k + 1) * KS + n1 * CL + ln] = cmul(z[k + 1], make_float2(w.z, w.w));
+        }
       }
     __syncthreads();  // the staging buffer is free: fetch the next item
     if (t == 0 && w + (int)gridDim.x < items) issue(w + gridDim.x);
@@ -261,13 +324,21 @@ __global__ void __launch_bounds__(P1 * P2, (P1 * P2 <= 320 ? 2 : 1))
         DFT<P1, -1>::run(y);
 #pragma unroll
         for (int k1 = 0; k1 < P1; ++k1) y[k1] = cscale(y[k1], __ldg(op.That + (size_t)(k2 + P2 * k1) * L + kx));
-        colb_inv_store<P1, P2, CL>(y, k2, ln, buf, tws);
+        DFT<P1, 1>::run(y);
+        colb_store<P1, P2, CL>(y, k2, ln, buf);
       }
       __syncthreads();
       for (int jj = t; jj < P1 * CL; jj += NT) {
         const int n1 = jj / CL, ln = jj - n1 * CL;
         float2 z[P2];
-        cola_load<P1, P2, 1, CL>(z, n1, ln, buf);
+#pragma unroll
+        for (int k = 0; k < P2; k += 2) {
+          const float4 w = *reinterpret_cast<const float4*>(tws + n1 * TS + k);
+          z[k] = buf[k * KS + n1 * CL + ln];
+          if (k > 0) z[k] = cmul_cb(z[k], make_float2(w.x, w.y));
+          z[k + 1] = cmul_cb(buf[(k + 1) * KS + n1 * CL + ln], make_float2(w.z, w.w));
+        }
+        DFT<P2, 1>::run(z);
 #pragma unroll
         for (int n2 = 0; n2 < NIN; ++n2) g[(size_t)(n1 + P1 * n2) * L + x0 + ln] = z[n2];  // rows < N only
       }
@@ -279,73 +350,155 @@ __global__ void __launch_bounds__(P1 * P2, (P1 * P2 <= 320 ? 2 : 1))
 // ---------------------------------------------------------------------------
 // Pass 3: rows: inverse FFT per coil, first N samples, conj(S) combine, + lam p
 // ---------------------------------------------------------------------------
-template <int P1, int P2, bool CG, bool PAD, int RL>
-__global__ void __launch_bounds__(RowSplit<P1, P2, RL>::NT, RowSplit<P1, P2, RL>::MINB)
-    k_toep_rows_inv(SpiralOp op, const float2* __restrict__ G, const float2* __restrict__ xin,
+// The grid rows of a step arrive by one TMA tensor load per coil, in the
+// swizzled exchange layout, and are transformed in place; those of the next
+// step are requested as soon as the a-jobs hold their last coil in registers.
+template <int P1, int P2, bool CG, bool PAD, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT)
+    k_toep_rows_inv(SpiralOp op, const __grid_constant__ CUtensorMap mG, const float2* __restrict__ xin,
                     float2* __restrict__ yout, float lam, CgArgs a, int it) {
+  using Rp = RowPass<P1, P2, NT>;
+  constexpr int RL = Rp::RL, CS = Rp::CS, GA = Rp::GA, CA = Rp::CA;
   constexpr int NIN = PAD ? P2 / 2 : P2;
   constexpr int L = P1 * P2;
-  constexpr int NT = RowSplit<P1, P2, RL>::NT;
+  constexpr int N = PAD ? L / 2 : L;
   extern __shared__ __align__(16) unsigned char smraw[];
-  float2* buf = reinterpret_cast<float2*>(smraw);
-  float2* tws = buf + RL * P2 * Split<P1, P2>::LD;
+  unsigned char* ex = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
+  float2* sst = reinterpret_cast<float2*>(ex + CS * Rp::slot);  // [CS][RL][N]
+  float2* twt = sst + CS * RL * N;                              // [P2][P1]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(twt + L);
   __shared__ double red[(NT + 31) / 32];
   __shared__ float sh_beta;
   __shared__ int sh_done;
-  const int t = threadIdx.x, b = blockIdx.y, N = op.n;
-  for (int i = t; i < L; i += NT) tws[i] = op.tw2[i];
+  const int t = threadIdx.x, b = blockIdx.y, y0 = blockIdx.x * RL;
+  if (t == 0) {
+    tc::mbar_init(bar, 1);
+    tc::mbar_init(bar + 1, 1);
+    tc::fence_mbar_init();
+  }
+  for (int i = t; i < L; i += NT) twt[i] = op.tw2[(i / P1) * (i % P1)];
   if (CG) cg_scalars(a, b, it, &sh_done, &sh_beta);
   __syncthreads();
   if (CG && sh_done) return;
+  auto issue_g = [&](int c0) {  // grid rows of a step
+    const int cn = min(CS, op.nc - c0);
+    tc::mbar_expect_tx(bar, (uint32_t)(cn * RL * L * 8));
+    for (int l = 0; l < cn * RL; ++l)
+      tc::tma_load_3d(ex + l * Rp::line, &mG, bar, 0, 0, (b * op.nc + c0 + l / RL) * N + y0 + l % RL);
+  };
+  auto issue_s = [&](int c0) {  // its sensitivity rows
+    const int cn = min(CS, op.nc - c0);
+    tc::mbar_expect_tx(bar + 1, (uint32_t)(cn * RL * N * 8));
+    for (int c = 0; c < cn; ++c)
+      tc::bulk_load(sst + c * RL * N, op.smaps + ((size_t)(c0 + c) * N + y0) * N, RL * N * 8, bar + 1);
+  };
+  if (t == 0) issue_g(0);
 
-  const int ra = t / P1, n1 = t % P1;
-  const bool ajob = t < RL * P1;
-  const int ya = blockIdx.x * RL + ra;
-  const bool aval = ajob && ya < N;
-  const int rb = t / P2, k2 = t % P2;
-  const bool bjob = t < RL * P2;
-  const int yb = blockIdx.x * RL + rb;
-  const bool bval = bjob && yb < N;
-  const size_t img = (size_t)b * N * N;
-
-  float2 acc[NIN];
+  const int g = t / (RL * P1), mm = t - g * (RL * P1), ra = mm / P1, n1 = mm - ra * P1;
+  const bool ajob = t < Rp::AT;
+  const int cb = t / (RL * P2), rb = (t / P2) % RL, k2 = t % P2;
+  // each a-thread owns NO image columns of its (row, n1); with several subgroups
+  // the owners add the coils' samples in coil order too, so that the sum's bits
+  // (and the p^H q partial's, summed as one thread per (row, n1) would) do not
+  // depend on the number of threads, that is on the batch
+  constexpr int NO = NIN / GA;
+  float2 acc[NO];
 #pragma unroll
-  for (int n2 = 0; n2 < NIN; ++n2) acc[n2] = make_float2(0.f, 0.f);
-  for (int c = 0; c < op.nc; ++c) {
-    if (bjob) {
-      float2 y[P1];
-      const float2* __restrict__ g = G + (((size_t)b * op.nc + c) * N + (bval ? yb : 0)) * L;
-#pragma unroll
-      for (int k1 = 0; k1 < P1; ++k1) y[k1] = bval ? g[k2 + P2 * k1] : make_float2(0.f, 0.f);
-      rowb_inv_store<P1, P2>(y, k2, rb, buf, tws);
+  for (int i = 0; i < NO; ++i) acc[i] = make_float2(0.f, 0.f);
+  bool ok = true;
+  int phase = 0;
+  for (int c0 = 0; c0 < op.nc; c0 += CS, phase ^= 1) {
+    if (ok && !tc::mbar_wait(bar, phase)) {  // reported by pico_sync; the block runs on so that its barriers pair up
+      ok = false;
+      if (op.err) atomicCAS(op.err, 0, 12);
     }
-    __syncthreads();
-    if (ajob) {
-      float2 z[P2];
-      rowa_inv_load<P1, P2>(z, n1, ra, buf);
-      if (aval) {
-        const float2* __restrict__ S = op.smaps + ((size_t)c * N + ya) * N;
+    if (c0 + cb < op.nc) {
+      float2 y[P1];
+      unsigned char* e = ex + cb * Rp::slot + rb * Rp::line;
 #pragma unroll
-        for (int n2 = 0; n2 < NIN; ++n2) acc[n2] = cfma_c(acc[n2], __ldg(S + n1 + P1 * n2), z[n2]);
+      for (int m = 0; m < P1; ++m) y[m] = *reinterpret_cast<const float2*>(e + Rp::at(m, k2));
+      DFT<P1, 1>::run(y);
+#pragma unroll
+      for (int m = 0; m < P1; ++m) *reinterpret_cast<float2*>(e + Rp::at(m, k2)) = y[m];
+    }
+    __syncthreads();  // rows transformed; the sensitivities of the step before were last read before it
+    if (t == 0) issue_s(c0);
+#pragma unroll 1
+    for (int j = 0; j < CA; ++j) {
+      const int cs = j * GA + g;
+      const bool on = ajob && c0 + cs < op.nc;
+      unsigned char* e = ex + cs * Rp::slot + ra * Rp::line;
+      float2 z[P2];
+      if (on) {
+#pragma unroll
+        for (int k = 0; k < P2; k += 2) {
+          const float4 v = *reinterpret_cast<const float4*>(e + Rp::at(n1, k));
+          z[k] = k == 0 ? make_float2(v.x, v.y) : cmul_cb(make_float2(v.x, v.y), twt[k * P1 + n1]);
+          z[k + 1] = cmul_cb(make_float2(v.z, v.w), twt[(k + 1) * P1 + n1]);
+        }
+      }
+      if (GA == 1 && j == CA - 1) {
+        tc::fence_proxy_async_smem();  // the in-place writes before the next step's copies
+        __syncthreads();               // the slots are free
+        if (t == 0 && c0 + CS < op.nc) issue_g(c0 + CS);
+      }
+      if (on) DFT<P2, 1>::run(z);
+      if (j == 0 && ok && !tc::mbar_wait(bar + 1, phase)) {
+        ok = false;
+        if (op.err) atomicCAS(op.err, 0, 12);
+      }
+      if (GA == 1) {
+        if (on) {
+          const float2* S = sst + (cs * RL + ra) * N + n1;
+#pragma unroll
+          for (int i = 0; i < NO; ++i) acc[i] = cfma_c(acc[i], S[P1 * i], z[i]);
+        }
+      } else if (on) {  // handed to the owners, in this job's own row
+#pragma unroll
+        for (int n2 = 0; n2 < NIN; n2 += 2)
+          *reinterpret_cast<float4*>(e + Rp::at(n1, n2)) = make_float4(z[n2].x, z[n2].y, z[n2 + 1].x, z[n2 + 1].y);
       }
     }
-    __syncthreads();
+    if (GA > 1) {
+      __syncthreads();
+      if (ajob) {
+        const int cn = min(CS, op.nc - c0);
+#pragma unroll 2
+        for (int cs = 0; cs < cn; ++cs) {
+          const unsigned char* e = ex + cs * Rp::slot + ra * Rp::line;
+          const float2* S = sst + (cs * RL + ra) * N + n1 + P1 * NO * g;
+#pragma unroll
+          for (int i = 0; i < NO; ++i)
+            acc[i] = cfma_c(acc[i], S[P1 * i], *reinterpret_cast<const float2*>(e + Rp::at(n1, NO * g + i)));
+        }
+      }
+      tc::fence_proxy_async_smem();
+      __syncthreads();
+      if (t == 0 && c0 + CS < op.nc) issue_g(c0 + CS);
+    }
   }
   float pq = 0.f;
-  if (aval) {
+  float* term = reinterpret_cast<float*>(ex);  // [RL P1][NIN] (GA > 1)
+  if (ajob) {
     const float2* __restrict__ pin = CG ? a.P : xin;
     float2* __restrict__ out = CG ? a.Q : yout;
 #pragma unroll
-    for (int n2 = 0; n2 < NIN; ++n2) {
-      const int x = n1 + P1 * n2;
-      {
-        const size_t idx = img + (size_t)ya * N + x;
-        const float2 pv = pin[idx];
-        const float2 q = make_float2(fmaf(lam, pv.x, acc[n2].x), fmaf(lam, pv.y, acc[n2].y));
-        out[idx] = q;
+    for (int i = 0; i < NO; ++i) {
+      const size_t idx = ((size_t)b * N + y0 + ra) * N + n1 + P1 * (NO * g + i);
+      const float2 pv = pin[idx];
+      const float2 q = make_float2(fmaf(lam, pv.x, acc[i].x), fmaf(lam, pv.y, acc[i].y));
+      out[idx] = q;
+      if (GA == 1)
         pq += cdot_re(pv, q);
-      }
+      else if (CG)
+        term[mm * NIN + NO * g + i] = cdot_re(pv, q);
     }
+  }
+  if (CG && GA > 1) {
+    __syncthreads();
+    if (t < RL * P1)
+#pragma unroll
+      for (int n2 = 0; n2 < NIN; ++n2) pq += term[t * NIN + n2];
   }
   if (CG) {
     const double tot = block_sum_d((double)pq, red);
@@ -478,94 +631,82 @@ __global__ void __launch_bounds__(Split<P1, P2>::NT, 1)
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-// Row passes of RL image rows per block (grid: ceil(n / RL) row blocks per
-// image; the p^H q partials of the inverse pass, one per row block, fill the
-// context's ceil(n / RL) slots).
-template <int P1, int P2, bool PAD, int RL>
+// Row passes (grid: n / RL row blocks per image; the p^H q partials of the
+// inverse pass, one per row block, fill the context's slots).
+template <int P1, int P2, bool PAD, int NT>
 void toep_rows_fwd_launch(const SpiralOp& op, const float2* x, float2* G, int nb, const CgArgs* a, int it,
                           cudaStream_t s) {
-  using Rs = RowSplit<P1, P2, RL>;
-  const size_t smr = Rs::buf + P1 * P2 * sizeof(float2);
-  const dim3 grow((op.n + RL - 1) / RL, nb);
-  if (a) {
-    auto k1 = k_toep_rows_fwd<P1, P2, true, PAD, RL>;
-    cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
-    k1<<<grow, Rs::NT, smr, s>>>(op, nullptr, G, *a, it);
-  } else {
-    CgArgs dummy{};
-    auto k1 = k_toep_rows_fwd<P1, P2, false, PAD, RL>;
-    cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
-    k1<<<grow, Rs::NT, smr, s>>>(op, x, G, dummy, 0);
-  }
+  using Rp = RowPass<P1, P2, NT>;
+  const size_t sm = Rp::smem(op.n);
+  const dim3 grow(op.n / Rp::RL, nb);
+  auto k1 = a ? k_toep_rows_fwd<P1, P2, true, PAD, NT> : k_toep_rows_fwd<P1, P2, false, PAD, NT>;
+  cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k1<<<grow, NT, sm, s>>>(op, x, G, a ? *a : CgArgs{}, it);
 }
-template <int P1, int P2, bool PAD, int RL>
-void toep_rows_inv_launch(const SpiralOp& op, const float2* x, float2* y, const float2* G, int nb, float lam,
+template <int P1, int P2, bool PAD, int NT>
+bool toep_rows_inv_launch(const SpiralOp& op, const float2* x, float2* y, const float2* G, int nb, float lam,
                           const CgArgs* a, int it, cudaStream_t s) {
-  using Rs = RowSplit<P1, P2, RL>;
-  const size_t smr = Rs::buf + P1 * P2 * sizeof(float2);
-  const dim3 grow((op.n + RL - 1) / RL, nb);
-  if (a) {
-    auto k3 = k_toep_rows_inv<P1, P2, true, PAD, RL>;
-    cudaFuncSetAttribute(k3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
-    k3<<<grow, Rs::NT, smr, s>>>(op, G, nullptr, nullptr, lam, *a, it);
-  } else {
-    CgArgs dummy{};
-    auto k3 = k_toep_rows_inv<P1, P2, false, PAD, RL>;
-    cudaFuncSetAttribute(k3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
-    k3<<<grow, Rs::NT, smr, s>>>(op, G, x, y, lam, dummy, 0);
-  }
+  using Rp = RowPass<P1, P2, NT>;
+  CUtensorMap mG{};
+  if (!encode_row_map(&mG, G, P1, P2, (int64_t)nb * op.nc * op.n, 1)) return false;
+  const size_t sm = Rp::smem(op.n);
+  const dim3 grow(op.n / Rp::RL, nb);
+  auto k3 = a ? k_toep_rows_inv<P1, P2, true, PAD, NT> : k_toep_rows_inv<P1, P2, false, PAD, NT>;
+  cudaFuncSetAttribute(k3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k3<<<grow, NT, sm, s>>>(op, mG, x, y, lam, a ? *a : CgArgs{}, it);
+  return true;
 }
 
 template <int P1, int P2, bool PAD>
-void toep_normal_impl(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam, const CgArgs* a,
+bool toep_cols_launch(const SpiralOp& op, float2* G, int nb, const int* done, int nsm, cudaStream_t s) {
+  using Cw = ColsW<P1, P2>;
+  CUtensorMap mG{};
+  const int box_rows = op.n <= 256 ? op.n : op.n / 2;  // TMA boxes of at most 256 rows
+  if (!encode_plane_map(&mG, G, op.n, P1 * P2, (int64_t)nb * op.nc, Cw::CL, box_rows)) return false;
+  auto k2 = k_toep_cols_w<P1, P2, PAD>;
+  const size_t sm = Cw::smem(op.n);
+  static thread_local int bps = 0;
+  cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (bps == 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k2, Cw::NT, sm) != cudaSuccess) bps = 1;
+  const int64_t items = (int64_t)(P1 * P2 / Cw::CL) * nb * op.nc;
+  const int grid = (int)std::min<int64_t>(items, (int64_t)std::max(1, bps) * nsm);
+  k2<<<grid, Cw::NT, sm, s>>>(op, mG, G, done, nb * op.nc, box_rows);
+  return true;
+}
+
+// Threads per block of the row passes: 128 (64 where the a-jobs of four rows fit
+// in 64), four (eight) blocks per SM, once the row blocks fill the device; below
+// that more coils at once per block, which shortens the serial walk over the
+// coils -- 256 threads while all blocks are resident at two per SM, 512 while
+// one per SM is enough.
+template <int P1, int P2, bool PAD, int NT>
+bool toep_normal_nt(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam, const CgArgs* a,
+                    int it, int nsm, cudaStream_t s) {
+  toep_rows_fwd_launch<P1, P2, PAD, NT>(op, x, G, nb, a, it, s);
+  return toep_cols_launch<P1, P2, PAD>(op, G, nb, a ? a->done : nullptr, nsm, s) &&
+         toep_rows_inv_launch<P1, P2, PAD, NT>(op, x, y, G, nb, lam, a, it, s);
+}
+
+template <int P1, int P2, bool PAD>
+bool toep_normal_impl(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam, const CgArgs* a,
                       int it, cudaStream_t s) {
-  using Sp = Split<P1, P2>;
-  constexpr int L = P1 * P2;
-  const size_t smc = Sp::col_buf + L * sizeof(float2);
-  if (op.row_lines == 4)
-    toep_rows_fwd_launch<P1, P2, PAD, 4>(op, x, G, nb, a, it, s);
-  else
-    toep_rows_fwd_launch<P1, P2, PAD, kLines>(op, x, G, nb, a, it, s);
-  // persistent column pass (P1 > P2): N rows staged per item, TMA boxes of at
-  // most 256 rows, every TMA destination 128-byte aligned
-  bool wide = false;
-  if constexpr (P1 > P2) {
-    const int box_rows = op.n <= 256 ? op.n : op.n / 2;
-    CUtensorMap mG{};
-    const size_t smw = 1024 + ((size_t)op.n * P1 + (size_t)L * P1 + L) * sizeof(float2) + 16;
-    wide = op.n % box_rows == 0 && ((size_t)box_rows * P1 * 8) % 128 == 0 && smw <= 227 * 1024 &&
-           encode_plane_map(&mG, G, op.n, L, (int64_t)nb * op.nc, P1, box_rows);
-    if (wide) {
-      auto k2 = k_toep_cols_w<P1, P2, PAD>;
-      static thread_local int bps = 0;
-      cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw);
-      if (bps == 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k2, L, smw) != cudaSuccess) bps = 1;
-      int dev = 0, nsm = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-      const int64_t items = (int64_t)P2 * nb * op.nc;
-      const int grid = (int)std::min<int64_t>(items, (int64_t)std::max(1, bps) * std::max(1, nsm));
-      k2<<<grid, L, smw, s>>>(op, mG, G, a ? a->done : nullptr, nb * op.nc, box_rows);
-    }
-  }
-  if (!wide) {
-    auto k2 = k_toep_cols<P1, P2, PAD>;
-    cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc);
-    k2<<<dim3(L / kLines, nb * op.nc), Sp::NT, smc, s>>>(op, G, a ? a->done : nullptr);
-  }
-  if (op.row_lines == 4)
-    toep_rows_inv_launch<P1, P2, PAD, 4>(op, x, y, G, nb, lam, a, it, s);
-  else
-    toep_rows_inv_launch<P1, P2, PAD, kLines>(op, x, y, G, nb, lam, a, it, s);
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  nsm = std::max(1, nsm);
+  const int64_t blocks = (int64_t)nb * (op.n / kRowLines);
+  constexpr bool wide = RowPass<P1, P2, 512>::smem(PAD ? P1 * P2 / 2 : P1 * P2) <= 227 * 1024;
+  if constexpr (wide)
+    if (blocks <= nsm) return toep_normal_nt<P1, P2, PAD, 512>(op, x, y, G, nb, lam, a, it, nsm, s);
+  if (blocks <= 2 * nsm) return toep_normal_nt<P1, P2, PAD, 256>(op, x, y, G, nb, lam, a, it, nsm, s);
+  return toep_normal_nt<P1, P2, PAD, (kRowLines * P1 <= 64 ? 64 : 128)>(op, x, y, G, nb, lam, a, it, nsm, s);
 }
 
 template <int P1, int P2>
-void launch_toep_normal_t(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam,
+bool launch_toep_normal_t(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam,
                           const CgArgs* a, int it, cudaStream_t s) {
-  if (op.L == 2 * op.n)
-    toep_normal_impl<P1, P2, true>(op, x, y, G, nb, lam, a, it, s);
-  else
-    toep_normal_impl<P1, P2, false>(op, x, y, G, nb, lam, a, it, s);
+  return op.L == 2 * op.n ? toep_normal_impl<P1, P2, true>(op, x, y, G, nb, lam, a, it, s)
+                          : toep_normal_impl<P1, P2, false>(op, x, y, G, nb, lam, a, it, s);
 }
 
 template <int P1, int P2>
