@@ -818,8 +818,15 @@ void cs_fista(pico_ctx* c, const float2* rhs, int64_t rhs_stride, int nb, bool k
   const float inv_lc = (float)(1.0 / c->cs_lc), tau = (float)c->cs_tau;
   cudaMemsetAsync(x, 0, (size_t)nb * n * sizeof(float2), c->stream);
   cudaMemsetAsync(z, 0, (size_t)nb * n * sizeof(float2), c->stream);
+  const bool fused = pico::cs_fused_supported(c->ny, c->cs_levels);
   for (int k = 0; k < c->cs_iters; ++k) {
     op_apply(c, z, t2, nb, 0.f);
+    if (fused) {
+      Launch L(c, 3, pico::cs_fused_kernels(c->ny, c->cs_levels));
+      pico::launch_cs_iter(z, t2, rhs, rhs_stride, inv_lc, nullptr, keep ? c->cs_traj + (size_t)k * n : nullptr, tau,
+                           t3, t2, x, z, c->cs_c[k], c->ny, c->cs_levels, nb, c->wav, c->stream);
+      continue;
+    }
     { Launch L(c, 3); pico::launch_cs_gradstep(z, t2, rhs, rhs_stride, inv_lc, t3, n, nb, c->stream); }
     cs_W(c, t3, t3, t2, nb, c->cs_levels);
     { Launch L(c, 3); pico::launch_cs_soft(t3, keep ? c->cs_traj + (size_t)k * n : nullptr, t3, tau, n, nb,
@@ -836,8 +843,15 @@ void cs_jvp_core(pico_ctx* c, const float2* ahdb, int nb) {
   const float inv_lc = (float)(1.0 / c->cs_lc), tau = (float)c->cs_tau;
   cudaMemsetAsync(dx, 0, (size_t)nb * n * sizeof(float2), c->stream);
   cudaMemsetAsync(dz, 0, (size_t)nb * n * sizeof(float2), c->stream);
+  const bool fused = pico::cs_fused_supported(c->ny, c->cs_levels);
   for (int k = 0; k < c->cs_iters; ++k) {
     op_apply(c, dz, t2, nb, 0.f);
+    if (fused) {
+      Launch L(c, 3, pico::cs_fused_kernels(c->ny, c->cs_levels));
+      pico::launch_cs_iter(dz, t2, ahdb, n, inv_lc, c->cs_traj + (size_t)k * n, nullptr, tau, t3, t2, dx, dz,
+                           c->cs_c[k], c->ny, c->cs_levels, nb, c->wav, c->stream);
+      continue;
+    }
     { Launch L(c, 3); pico::launch_cs_gradstep(dz, t2, ahdb, n, inv_lc, t3, n, nb, c->stream); }
     cs_W(c, t3, t3, t2, nb, c->cs_levels);
     { Launch L(c, 3); pico::launch_cs_soft_tan(c->cs_traj + (size_t)k * n, t3, tau, n, nb, c->stream); }
@@ -853,6 +867,21 @@ void cs_vjp_core(pico_ctx* c, const float2* xbar, int nb) {
   const float inv_lc = (float)(1.0 / c->cs_lc), tau = (float)c->cs_tau;
   cudaMemsetAsync(ys, 0, (size_t)nb * n * sizeof(float2), c->stream);
   cudaMemsetAsync(zb, 0, (size_t)nb * n * sizeof(float2), c->stream);
+  if (pico::cs_fused_supported(c->ny, c->cs_levels)) {
+    // z alternates between two buffers: a tile's halo reads the old one
+    float2 *yb = cs_e(c, 4), *zc[2] = {zb, xbn};
+    for (int k = c->cs_iters - 1, i = 0; k >= 0; --k, ++i) {
+      {
+        Launch L(c, 3, pico::cs_fused_kernels(c->ny, c->cs_levels));
+        pico::launch_vjp_iter(i ? yb : nullptr, t2, inv_lc, i ? zc[(i + 1) & 1] : xbar, i ? c->cs_c[k + 1] : 0.f,
+                              c->cs_c[k], zc[i & 1], c->cs_traj + (size_t)k * n, tau, t3, t2, yb, ys, c->ny,
+                              c->cs_levels, nb, c->wav, c->stream);
+      }
+      if (k > 0) op_apply(c, yb, t2, nb, 0.f);  // the last M yb would only feed a z that nothing reads
+    }
+    Launch L(c, 3);
+    return pico::launch_scale(ys, inv_lc, n, nb, c->stream);
+  }
   cudaMemcpyAsync(xbn, xbar, (size_t)nb * n * sizeof(float2), cudaMemcpyDeviceToDevice, c->stream);
   for (int k = c->cs_iters - 1; k >= 0; --k) {
     { Launch L(c, 3); pico::launch_vjp_a(xbn, zb, t3, c->cs_c[k], n, nb, c->stream); }

@@ -108,13 +108,15 @@ __global__ void k_copy_region(const float2* __restrict__ in, float2* __restrict_
 }
 
 // ---- element-wise FISTA / Jacobian steps (image index i, batch b = blockIdx.y) ----
+// |c|, the one rounding order written out so that every kernel that inlines it agrees
+__device__ __forceinline__ float cs_abs(float2 c) { return sqrtf(fmaf(c.x, c.x, __fmul_rn(c.y, c.y))); }
 __device__ __forceinline__ float2 soft1(float2 c, float tau) {
-  const float a = sqrtf(c.x * c.x + c.y * c.y);
+  const float a = cs_abs(c);
   if (!(a > tau)) return make_float2(0.f, 0.f);
   return cscale(c, 1.f - tau / a);
 }
 __device__ __forceinline__ float2 soft_tan1(float2 c, float tau, float2 dc) {
-  const float a = sqrtf(c.x * c.x + c.y * c.y);
+  const float a = cs_abs(c);
   if (!(a > tau)) return make_float2(0.f, 0.f);
   const float2 u = cscale(c, 1.f / a);
   const float re = cdot_re(u, dc);  // Re(conj(u) dc)
@@ -122,6 +124,8 @@ __device__ __forceinline__ float2 soft_tan1(float2 c, float tau, float2 dc) {
   return make_float2(fmaf(s, dc.x, q * u.x), fmaf(s, dc.y, q * u.y));
 }
 
+// The element-wise steps as passes of their own: for transforms whose last
+// levels are shorter than the filter (cs_fused_supported).
 // y = z - (Mz - rhs) / Lc ; rhs broadcast when rhs_stride == 0
 __global__ void k_cs_gradstep(const float2* __restrict__ z, const float2* __restrict__ Mz,
                               const float2* __restrict__ rhs, int64_t rhs_stride, float inv_lc, float2* __restrict__ y,
@@ -143,15 +147,6 @@ __global__ void k_cs_soft(const float2* c, float2* __restrict__ keep, float2* ou
   const float2 v = c[o];
   if (keep) keep[i] = v;
   out[o] = soft1(v, tau);
-}
-
-// x[b] += alpha y (y one image, broadcast over the batch)
-__global__ void k_axpy_bcast(float2* __restrict__ x, const float2* __restrict__ y, float alpha, int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const size_t o = (size_t)blockIdx.y * n + i;
-  const float2 a = x[o], b = y[i];
-  x[o] = make_float2(fmaf(alpha, b.x, a.x), fmaf(alpha, b.y, a.y));
 }
 
 // tangent of the soft threshold at the stored coefficients (broadcast over the batch), in place
@@ -194,6 +189,343 @@ __global__ void k_vjp_b(const float2* __restrict__ yb, const float2* __restrict_
   zb[o] = make_float2(fmaf(-inv_lc, m.x, y.x), fmaf(-inv_lc, m.y, y.y));
   const float2 s = ysum[o];
   ysum[o] = make_float2(s.x + y.x, s.y + y.y);
+}
+
+// x[b] += alpha y (y one image, broadcast over the batch)
+__global__ void k_axpy_bcast(float2* __restrict__ x, const float2* __restrict__ y, float alpha, int64_t n) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const size_t o = (size_t)blockIdx.y * n + i;
+  const float2 a = x[o], b = y[i];
+  x[o] = make_float2(fmaf(alpha, b.x, a.x), fmaf(alpha, b.y, a.y));
+}
+
+// ---------------------------------------------------------------------------
+// One FISTA / tangent / adjoint iteration around the normal operator, fused:
+//   cs_fwd    (level 0)  iteration step on load, 2-D analysis, threshold of the finished coefficients
+//   cs_fwd    (level l)  2-D analysis of the approximation band, threshold
+//   cs_core              the remaining levels of one image in shared memory: analysis, threshold, synthesis
+//   cs_inv    (level l)  2-D synthesis
+//   cs_inv    (level 0)  2-D synthesis, iteration step on store
+// instead of one launch per direction and level and one per element-wise step:
+// 5 launches per iteration of a 4-level transform at 320 x 320 in place of
+// 19-20, the images cross memory once per level and direction instead of twice,
+// and the element-wise steps take no pass of their own (320 x 320, 48 images:
+// 367 us of such passes per iteration before, 205 us as fused; one image: 84 us
+// before).  The arithmetic of every value is that of the
+// single passes (rows before columns in the analysis, columns before rows in the
+// synthesis, taps in the same order).  Bound by the loads of the level-0
+// kernels (L2 / HBM) for many images and by the launches for one.
+// ---------------------------------------------------------------------------
+constexpr int kTapMax = 8;
+constexpr int kFuseTX = 32;        // coefficients per tile and band along x
+constexpr int kFuseThreads = 256;
+
+struct FwdArgs {
+  int n, m;                        // image side, side of this level's input region
+  const float2 *a, *b, *c;         // load operands (see cs_load)
+  int64_t c_stride;                // image stride of c (0: one image for the whole batch)
+  float s0, s1, s2;
+  float2* zout;                    // kLoadVjp: the new z, stored by the tile that owns the pixel
+  float2* dst;
+  const float2* at;                // threshold tangent: stored coefficients (one image)
+  float2* keep;                    // primal: raw coefficients kept (one image), or nullptr
+  float tau;
+  int last;                        // the approximation band is finished too
+};
+enum { kLoadGrad, kLoadVjp, kLoadPlain };
+
+// kLoadGrad:  a - (b - c) s0            (y = z - (M z - rhs) / Lc)
+// kLoadVjp:   z = a - b s0 (0 if !a);  c' = a ? -s2 c : c;  c' + s1 z
+//             (reverse sweep: zb = yb - M yb / Lc, xk = xb + (1 + c_k) zb with xb = -c_{k+1} zb_prev)
+template <int LOAD>
+__device__ __forceinline__ float2 cs_load(const FwdArgs& f, size_t o, size_t i, int b, bool own) {
+  if (LOAD == kLoadPlain) return f.a[o];
+  if (LOAD == kLoadGrad) {
+    const float2 z = f.a[o], mz = f.b[o], r = f.c[(size_t)b * f.c_stride + i];
+    return make_float2(fmaf(-f.s0, mz.x - r.x, z.x), fmaf(-f.s0, mz.y - r.y, z.y));
+  }
+  float2 z = make_float2(0.f, 0.f), xb = f.c[o];
+  if (f.a) {
+    const float2 y = f.a[o], my = f.b[o];
+    z = make_float2(fmaf(-f.s0, my.x, y.x), fmaf(-f.s0, my.y, y.y));
+    xb = make_float2(-f.s2 * xb.x, -f.s2 * xb.y);
+  }
+  if (own) f.zout[o] = z;
+  return make_float2(fmaf(f.s1, z.x, xb.x), fmaf(f.s1, z.y, xb.y));
+}
+
+template <bool TAN>
+__device__ __forceinline__ float2 cs_threshold(float2 v, size_t i, const float2* at, float2* keep, float tau) {
+  if (TAN) return soft_tan1(at[i], tau, v);
+  if (keep) keep[i] = v;
+  return soft1(v, tau);
+}
+
+// One analysis level on tiles of TY x kFuseTX coefficients per band.
+template <int LOAD, bool TAN, int TY>
+__global__ void __launch_bounds__(kFuseThreads) k_cs_fwd(FwdArgs f, Wavelet w) {
+  constexpr int TX = kFuseTX, IY = 2 * TY + kTapMax - 2, IX = 2 * TX + kTapMax - 2;
+  __shared__ __align__(16) float2 in[IY][IX];
+  __shared__ float2 mid[IY][2 * TX];   // row analysis: [approximation | detail]
+  const int t = threadIdx.x, b = blockIdx.z, n = f.n, m = f.m, half = m / 2;
+  const int kx0 = blockIdx.x * TX, ky0 = blockIdx.y * TY;
+  const size_t img = (size_t)b * n * n;
+  for (int e = t; e < IY * IX; e += kFuseThreads) {
+    const int r = e / IX, q = e - r * IX;
+    int y = 2 * ky0 + r, x = 2 * kx0 + q;
+    const bool own = r < 2 * TY && q < 2 * TX && y < m && x < m;
+    // the last tile's overhang beyond the periodic halo is loaded from a valid place and not used
+    if (y >= m) y -= m;
+    if (x >= m) x -= m;
+    y = min(y, m - 1);
+    x = min(x, m - 1);
+    const size_t i = (size_t)y * n + x;
+    in[r][q] = cs_load<LOAD>(f, img + i, i, b, own);
+  }
+  __syncthreads();
+  for (int e = t; e < IY * TX; e += kFuseThreads) {
+    const int r = e / TX, k = e - r * TX;
+    float2 a = make_float2(0.f, 0.f), d = a;
+#pragma unroll
+    for (int q = 0; q < kTapMax; q += 2) {   // two values per access: no bank conflicts
+      const float4 v = *reinterpret_cast<const float4*>(&in[r][2 * k + q]);
+      a.x = fmaf(w.h[q], v.x, a.x);
+      a.y = fmaf(w.h[q], v.y, a.y);
+      d.x = fmaf(w.g[q], v.x, d.x);
+      d.y = fmaf(w.g[q], v.y, d.y);
+      a.x = fmaf(w.h[q + 1], v.z, a.x);
+      a.y = fmaf(w.h[q + 1], v.w, a.y);
+      d.x = fmaf(w.g[q + 1], v.z, d.x);
+      d.y = fmaf(w.g[q + 1], v.w, d.y);
+    }
+    mid[r][k] = a;
+    mid[r][TX + k] = d;
+  }
+  __syncthreads();
+  for (int e = t; e < TY * 2 * TX; e += kFuseThreads) {
+    const int k = e / (2 * TX), q0 = e - k * (2 * TX);
+    const int ky = ky0 + k, kx = kx0 + (q0 & (TX - 1)), band = q0 >= TX;
+    if (ky >= half || kx >= half) continue;
+    float2 a = make_float2(0.f, 0.f), d = a;
+#pragma unroll
+    for (int q = 0; q < kTapMax; ++q) {
+      const float2 v = mid[2 * k + q][q0];
+      a.x = fmaf(w.h[q], v.x, a.x);
+      a.y = fmaf(w.h[q], v.y, a.y);
+      d.x = fmaf(w.g[q], v.x, d.x);
+      d.y = fmaf(w.g[q], v.y, d.y);
+    }
+    const size_t ia = (size_t)ky * n + kx + band * half, id = ia + (size_t)half * n;
+    f.dst[img + ia] = (band || f.last) ? cs_threshold<TAN>(a, ia, f.at, f.keep, f.tau) : a;
+    f.dst[img + id] = cs_threshold<TAN>(d, id, f.at, f.keep, f.tau);
+  }
+}
+
+struct InvArgs {
+  int n, m;
+  const float2* src;   // all bands of the level, [m][m] of an n-strided image
+  float2 *o0, *o1;     // plain: o0 (n-strided); step: see cs_store
+  float c;
+};
+enum { kStorePlain, kStoreMomentum, kStoreVjp };
+
+// kStoreMomentum: z = v + c (v - x); x = v       (o0 = x, o1 = z)
+// kStoreVjp:      yb = v; ysum += v              (o0 = yb, o1 = ysum)
+template <int STORE>
+__device__ __forceinline__ void cs_store(const InvArgs& f, size_t o, float2 v) {
+  if (STORE == kStoreMomentum) {
+    const float2 x = f.o0[o];
+    f.o1[o] = make_float2(fmaf(f.c, v.x - x.x, v.x), fmaf(f.c, v.y - x.y, v.y));
+  } else if (STORE == kStoreVjp) {
+    const float2 s = f.o1[o];
+    f.o1[o] = make_float2(s.x + v.x, s.y + v.y);
+  }
+  f.o0[o] = v;
+}
+
+// One synthesis level on tiles of 2 TY x 2 kFuseTX outputs.
+template <int STORE, int TY>
+__global__ void __launch_bounds__(kFuseThreads) k_cs_inv(InvArgs f, Wavelet w) {
+  constexpr int TX = kFuseTX, HB = kTapMax / 2 - 1, CY = TY + HB, CX = TX + HB;
+  __shared__ float2 in[2][CY][2 * CX];     // [rows: approximation | detail][k][columns: approximation | detail]
+  __shared__ float2 mid[2 * TY][2 * CX];   // column synthesis
+  const int t = threadIdx.x, b = blockIdx.z, n = f.n, m = f.m, half = m / 2;
+  const int kx0 = blockIdx.x * TX, ky0 = blockIdx.y * TY;   // first own coefficient of the tile
+  const size_t img = (size_t)b * n * n;
+  for (int e = t; e < 2 * CY * 2 * CX; e += kFuseThreads) {
+    const int hy = e / (CY * 2 * CX), r = (e / (2 * CX)) % CY, q = e % (2 * CX), hx = q >= CX;
+    int ky = ky0 + r - HB, kx = kx0 + (q - hx * CX) - HB;
+    if (ky < 0) ky += half;
+    if (kx < 0) kx += half;
+    ky = min(ky, half - 1);
+    kx = min(kx, half - 1);
+    in[hy][r][q] = f.src[img + (size_t)(ky + hy * half) * n + kx + hx * half];
+  }
+  __syncthreads();
+  for (int e = t; e < 2 * TY * 2 * CX; e += kFuseThreads) {
+    const int i = e / (2 * CX), q = e - i * (2 * CX);
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kTapMax / 2; ++u) {   // tap q0 = 2 u + (i & 1), coefficient (i - q0) / 2
+      const int tap = 2 * u + (i & 1), k = (i >> 1) - u + HB;
+      const float2 a = in[0][k][q], d = in[1][k][q];
+      acc.x = fmaf(w.h[tap], a.x, fmaf(w.g[tap], d.x, acc.x));
+      acc.y = fmaf(w.h[tap], a.y, fmaf(w.g[tap], d.y, acc.y));
+    }
+    mid[i][q] = acc;
+  }
+  __syncthreads();
+  for (int e = t; e < 2 * TY * 2 * TX; e += kFuseThreads) {
+    const int r = e / (2 * TX), i = e - r * (2 * TX);
+    const int y = 2 * ky0 + r, x = 2 * kx0 + i;
+    if (y >= m || x >= m) continue;
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kTapMax / 2; ++u) {
+      const int tap = 2 * u + (i & 1), k = (i >> 1) - u + HB;
+      const float2 a = mid[r][k], d = mid[r][CX + k];
+      acc.x = fmaf(w.h[tap], a.x, fmaf(w.g[tap], d.x, acc.x));
+      acc.y = fmaf(w.h[tap], a.y, fmaf(w.g[tap], d.y, acc.y));
+    }
+    cs_store<STORE>(f, img + (size_t)y * n + x, acc);
+  }
+}
+
+// The last levels of one image (side m at the first of them, at most kCoreSide)
+// in shared memory: each pass reads one buffer and writes the other, rows with
+// consecutive lanes along the row, columns with consecutive lanes across them.
+// A latency-bound chain of 4 passes per level: 1024 threads, one (approximation,
+// detail) pair or one sample each and a barrier per pass.
+constexpr int kCoreSide = 96;
+constexpr int kCoreThreads = 1024;
+
+// taps along a line of `len` values (value x at p[x * st]): coefficient pair k
+__device__ __forceinline__ void core_pair(const float2* p, int st, int k, int len, const Wavelet& w, float2& oa,
+                                          float2& od) {
+  float2 a = make_float2(0.f, 0.f), d = a;
+#pragma unroll
+  for (int q = 0; q < kTapMax; ++q) {
+    int x = 2 * k + q;
+    if (x >= len) x -= len;
+    const float2 v = p[x * st];
+    a.x = fmaf(w.h[q], v.x, a.x);
+    a.y = fmaf(w.h[q], v.y, a.y);
+    d.x = fmaf(w.g[q], v.x, d.x);
+    d.y = fmaf(w.g[q], v.y, d.y);
+  }
+  oa = a;
+  od = d;
+}
+// samples 2 j and 2 j + 1 of a line from its [approximation | detail]
+__device__ __forceinline__ void core_samples(const float2* p, int st, int j, int half, const Wavelet& w, float2& oe,
+                                             float2& oo) {
+  float2 e = make_float2(0.f, 0.f), o = e;
+#pragma unroll
+  for (int u = 0; u < kTapMax / 2; ++u) {
+    int k = j - u;
+    if (k < 0) k += half;
+    const float2 a = p[k * st], d = p[(half + k) * st];
+    e.x = fmaf(w.h[2 * u], a.x, fmaf(w.g[2 * u], d.x, e.x));
+    e.y = fmaf(w.h[2 * u], a.y, fmaf(w.g[2 * u], d.y, e.y));
+    o.x = fmaf(w.h[2 * u + 1], a.x, fmaf(w.g[2 * u + 1], d.x, o.x));
+    o.y = fmaf(w.h[2 * u + 1], a.y, fmaf(w.g[2 * u + 1], d.y, o.y));
+  }
+  oe = e;
+  oo = o;
+}
+
+template <bool TAN>
+__global__ void __launch_bounds__(kCoreThreads) k_cs_core(float2* data, int n, int m, int levels, const float2* at,
+                                                          float2* keep, float tau, Wavelet w) {
+  extern __shared__ float2 core[];
+  float2 *A = core, *B = core + m * m;
+  float2* img = data + (size_t)blockIdx.x * n * n;
+  const int t = threadIdx.x;
+  for (int e = t; e < m * m; e += kCoreThreads) A[e] = img[(size_t)(e / m) * n + e % m];
+  __syncthreads();
+  for (int l = 0; l < levels; ++l) {
+    const int s = m >> l, half = s / 2;
+    for (int e = t; e < s * half; e += kCoreThreads) {
+      const int y = e / half, k = e - y * half;
+      core_pair(A + y * m, 1, k, s, w, B[y * m + k], B[y * m + half + k]);
+    }
+    __syncthreads();
+    for (int e = t; e < s * half; e += kCoreThreads) {
+      const int k = e / s, x = e - k * s;
+      core_pair(B + x, m, k, s, w, A[k * m + x], A[(half + k) * m + x]);
+    }
+    __syncthreads();
+  }
+  for (int e = t; e < m * m; e += kCoreThreads) {
+    const size_t i = (size_t)(e / m) * n + e % m;
+    A[e] = cs_threshold<TAN>(A[e], i, at, keep, tau);
+  }
+  __syncthreads();
+  for (int l = levels - 1; l >= 0; --l) {
+    const int s = m >> l, half = s / 2;
+    for (int e = t; e < s * half; e += kCoreThreads) {
+      const int j = e / s, x = e - j * s;
+      core_samples(A + x, m, j, half, w, B[2 * j * m + x], B[(2 * j + 1) * m + x]);
+    }
+    __syncthreads();
+    for (int e = t; e < s * half; e += kCoreThreads) {
+      const int y = e / half, j = e - y * half;
+      core_samples(B + y * m, 1, j, half, w, A[y * m + 2 * j], A[y * m + 2 * j + 1]);
+    }
+    __syncthreads();
+  }
+  for (int e = t; e < m * m; e += kCoreThreads) img[(size_t)(e / m) * n + e % m] = A[e];
+}
+
+template <int LOAD, bool TAN>
+void fwd_level(const FwdArgs& f, int nb, const Wavelet& w, cudaStream_t s) {
+  const int half = f.m / 2, bx = (half + kFuseTX - 1) / kFuseTX;
+  // tiles of 16 coefficient rows (halo 1.3x) once they fill the device, else of 8 (1.5x, twice the blocks)
+  if ((int64_t)bx * ((half + 15) / 16) * nb >= 1024)
+    k_cs_fwd<LOAD, TAN, 16><<<dim3(bx, (half + 15) / 16, nb), kFuseThreads, 0, s>>>(f, w);
+  else
+    k_cs_fwd<LOAD, TAN, 8><<<dim3(bx, (half + 7) / 8, nb), kFuseThreads, 0, s>>>(f, w);
+}
+template <int STORE>
+void inv_level(const InvArgs& f, int nb, const Wavelet& w, cudaStream_t s) {
+  const int half = f.m / 2, bx = (half + kFuseTX - 1) / kFuseTX;
+  if ((int64_t)bx * ((half + 15) / 16) * nb >= 1024)
+    k_cs_inv<STORE, 16><<<dim3(bx, (half + 15) / 16, nb), kFuseThreads, 0, s>>>(f, w);
+  else
+    k_cs_inv<STORE, 8><<<dim3(bx, (half + 7) / 8, nb), kFuseThreads, 0, s>>>(f, w);
+}
+
+// Coefficients of y (from cs_load<LOAD>) thresholded and transformed back:
+// analysis level 0 from the load operands into b0, further levels alternating
+// between b1 and b0, the small levels in place, synthesis up to level 1.
+// The thresholded level-0 bands end in b0.
+template <int LOAD, bool TAN>
+void cs_shrink(FwdArgs f, float2* b0, float2* b1, int levels, int nb, const Wavelet& w, cudaStream_t s) {
+  const int n = f.n;
+  float2* buf[2] = {b0, b1};
+  int l0 = 1;   // first level of the in-memory core
+  while (l0 < levels && (n >> l0) > kCoreSide) ++l0;
+  f.m = n;
+  f.dst = b0;
+  f.last = levels == 1;
+  fwd_level<LOAD, TAN>(f, nb, w, s);
+  for (int l = 1; l < l0; ++l) {
+    f.a = buf[(l - 1) & 1];
+    f.dst = buf[l & 1];
+    f.m = n >> l;
+    f.last = l == levels - 1;
+    fwd_level<kLoadPlain, TAN>(f, nb, w, s);
+  }
+  if (l0 < levels) {
+    const int m = n >> l0;
+    const size_t sm = (size_t)2 * m * m * sizeof(float2);
+    auto k = k_cs_core<TAN>;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k<<<nb, kCoreThreads, sm, s>>>(buf[(l0 - 1) & 1], n, m, levels - l0, f.at, f.keep, f.tau, w);
+  }
+  for (int l = l0 - 1; l >= 1; --l)
+    inv_level<kStorePlain>(InvArgs{n, n >> l, buf[l & 1], buf[(l - 1) & 1], nullptr, 0.f}, nb, w, s);
 }
 
 __global__ void k_scale(float2* __restrict__ x, float s, int64_t n) {
@@ -265,15 +597,15 @@ void launch_idwt(const float2* coef, float2* x, float2* tmp, int n, int levels, 
 int dwt_kernels(int levels) { return 2 * levels; }
 int idwt_kernels(int levels, bool in_place) { return 2 * levels + (in_place ? 0 : 1); }
 
+void launch_axpy_bcast(float2* x, const float2* y, float alpha, int64_t n, int nb, cudaStream_t s) {
+  k_axpy_bcast<<<dim3(blocks(n), nb), 256, 0, s>>>(x, y, alpha, n);
+}
 void launch_cs_gradstep(const float2* z, const float2* Mz, const float2* rhs, int64_t rhs_stride, float inv_lc,
                         float2* y, int64_t n, int nb, cudaStream_t s) {
   k_cs_gradstep<<<dim3(blocks(n), nb), 256, 0, s>>>(z, Mz, rhs, rhs_stride, inv_lc, y, n);
 }
 void launch_cs_soft(const float2* c, float2* keep, float2* out, float tau, int64_t n, int nb, cudaStream_t s) {
   k_cs_soft<<<dim3(blocks(n), nb), 256, 0, s>>>(c, keep, out, tau, n);
-}
-void launch_axpy_bcast(float2* x, const float2* y, float alpha, int64_t n, int nb, cudaStream_t s) {
-  k_axpy_bcast<<<dim3(blocks(n), nb), 256, 0, s>>>(x, y, alpha, n);
 }
 void launch_cs_soft_tan(const float2* at, float2* dc, float tau, int64_t n, int nb, cudaStream_t s) {
   k_cs_soft_tan<<<dim3(blocks(n), nb), 256, 0, s>>>(at, dc, tau, n);
@@ -287,6 +619,31 @@ void launch_vjp_a(float2* xbn, const float2* zb, float2* xk1, float c, int64_t n
 void launch_vjp_b(const float2* yb, const float2* Myb, float inv_lc, float2* zb, float2* ysum, int64_t n, int nb,
                   cudaStream_t s) {
   k_vjp_b<<<dim3(blocks(n), nb), 256, 0, s>>>(yb, Myb, inv_lc, zb, ysum, n);
+}
+bool cs_fused_supported(int n, int levels) { return levels >= 1 && (n >> (levels - 1)) >= kTapMax - 2; }
+int cs_fused_kernels(int n, int levels) {
+  int l0 = 1;
+  while (l0 < levels && (n >> l0) > kCoreSide) ++l0;
+  return 2 * l0 + (l0 < levels ? 1 : 0);
+}
+
+void launch_cs_iter(const float2* z, const float2* Mz, const float2* rhs, int64_t rhs_stride, float inv_lc,
+                    const float2* at, float2* keep, float tau, float2* b0, float2* b1, float2* x, float2* zout,
+                    float c, int n, int levels, int nb, const Wavelet& w, cudaStream_t s) {
+  FwdArgs f{n, n, z, Mz, rhs, rhs_stride, inv_lc, 0.f, 0.f, nullptr, b0, at, keep, tau, 0};
+  if (at)
+    cs_shrink<kLoadGrad, true>(f, b0, b1, levels, nb, w, s);
+  else
+    cs_shrink<kLoadGrad, false>(f, b0, b1, levels, nb, w, s);
+  inv_level<kStoreMomentum>(InvArgs{n, n, b0, x, zout, c}, nb, w, s);
+}
+
+void launch_vjp_iter(const float2* yb, const float2* Myb, float inv_lc, const float2* xb, float c_prev, float c,
+                     float2* znew, const float2* at, float tau, float2* b0, float2* b1, float2* yout, float2* ysum,
+                     int n, int levels, int nb, const Wavelet& w, cudaStream_t s) {
+  FwdArgs f{n, n, yb, Myb, xb, 0, inv_lc, 1.f + c, c_prev, znew, b0, at, nullptr, tau, 0};
+  cs_shrink<kLoadVjp, true>(f, b0, b1, levels, nb, w, s);
+  inv_level<kStoreVjp>(InvArgs{n, n, b0, yout, ysum, 0.f}, nb, w, s);
 }
 void launch_scale(float2* x, float sc, int64_t n, int nb, cudaStream_t s) {
   k_scale<<<dim3(blocks(n), nb), 256, 0, s>>>(x, sc, n);

@@ -273,6 +273,22 @@ void launch_idwt(const float2* coef, float2* x, float2* tmp, int n, int levels, 
                  cudaStream_t s);
 int dwt_kernels(int levels);
 int idwt_kernels(int levels, bool in_place);
+// Fused iterations (levels whose sides are at least the filter length less two):
+// one FISTA / tangent iteration around the normal operator,
+//   y = z - (M z - rhs) / Lc;  v = W^H S(W y);  zout = v + c (v - x);  x = v,
+// S the soft threshold, or with `at` its tangent at those coefficients; `keep`
+// receives the raw W y.  b0, b1: coefficient scratch; Mz may be b1.
+bool cs_fused_supported(int n, int levels);
+int cs_fused_kernels(int n, int levels);
+void launch_cs_iter(const float2* z, const float2* Mz, const float2* rhs, int64_t rhs_stride, float inv_lc,
+                    const float2* at, float2* keep, float tau, float2* b0, float2* b1, float2* x, float2* zout,
+                    float c, int n, int levels, int nb, const Wavelet& w, cudaStream_t s);
+// one reverse-sweep iteration: znew = yb - M yb / Lc (0 without yb), then
+//   yout = W^H S'(W (xb' + (1 + c) znew)), ysum += yout,
+// xb' = -c_prev xb (xb: the previous iteration's z), or xb itself without yb
+void launch_vjp_iter(const float2* yb, const float2* Myb, float inv_lc, const float2* xb, float c_prev, float c,
+                     float2* znew, const float2* at, float tau, float2* b0, float2* b1, float2* yout, float2* ysum,
+                     int n, int levels, int nb, const Wavelet& w, cudaStream_t s);
 void launch_cs_gradstep(const float2* z, const float2* Mz, const float2* rhs, int64_t rhs_stride, float inv_lc,
                         float2* y, int64_t n, int nb, cudaStream_t s);
 void launch_cs_soft(const float2* c, float2* keep, float2* out, float tau, int64_t n, int nb, cudaStream_t s);
