@@ -131,13 +131,16 @@ __global__ void __launch_bounds__(kVecThreads) k_cg_update(CgArgs a, int it) {
 }
 
 // Per-system CG step of iteration it, once per system: state 0 update,
-// 1 converged / stopped, 2 breakdown; alpha = rr / pq.
-__global__ void k_cg_alpha(CgArgs a, int it, float* alpha, int* state) {
-  const int b = blockIdx.x;
-  const double rr = warp_sum_parts(rr_at(a, b, it), a.PB);
-  const double rr0 = warp_sum_parts(rr_at(a, b, 0), a.PB);
-  const double pq = warp_sum_parts(pq_at(a, b, it), a.PA);
+// 1 converged / stopped, 2 breakdown; alpha = rr / pq.  Three warps, one sum each.
+__global__ void __launch_bounds__(96) k_cg_alpha(CgArgs a, int it, float* alpha, int* state) {
+  __shared__ double sum[3];
+  const int b = blockIdx.x, w = threadIdx.x >> 5;
+  const double* p = w == 0 ? pq_at(a, b, it) : rr_at(a, b, w == 1 ? it : 0);
+  const double v = warp_sum_parts_long(p, w == 0 ? a.PA : a.PB);
+  if ((threadIdx.x & 31) == 0) sum[w] = v;
+  __syncthreads();
   if (threadIdx.x == 0) {
+    const double pq = sum[0], rr = sum[1], rr0 = sum[2];
     state[b] = cg_state_of(rr, rr0, pq, a.rtol2);
     alpha[b] = (float)(rr / pq);
   }
@@ -425,14 +428,14 @@ void launch_cg_update(const CgArgs& a, int nb, int it, cudaStream_t s) {
 }
 bool launch_cg_step(const CgArgs& a, int nb, int it, float* alpha, int* state, cudaStream_t s) {
   if (a.n % 2) return false;
-  k_cg_alpha<<<nb, 32, 0, s>>>(a, it, alpha, state);
+  k_cg_alpha<<<nb, 96, 0, s>>>(a, it, alpha, state);
   k_cg_update_v<<<dim3(a.PB, nb), kVecThreads, 0, s>>>(a, it, alpha, state);
   return true;
 }
 bool launch_cg_step_pair(const CgArgs& a, int nb, int it, float* alpha, int* state, const float* alpha_prev,
                          const int* state_prev, const float2* p_prev, cudaStream_t s) {
   if (a.n % 2) return false;
-  k_cg_alpha<<<nb, 32, 0, s>>>(a, it, alpha, state);
+  k_cg_alpha<<<nb, 96, 0, s>>>(a, it, alpha, state);
   k_cg_update_pair<<<dim3(a.PB, nb), kVecThreads, 0, s>>>(a, it, alpha, state, alpha_prev, state_prev, p_prev,
                                                           it & 1);
   return true;

@@ -195,13 +195,18 @@ __global__ void __launch_bounds__(256) k_gram_build_smem(const float2* __restric
 // per-image CG scalars of iteration it: beta = rr(it) / rr(it-1) (0 at it = 0),
 // done flag, and the bound pn on the new direction's entries (|p| <= ||p|| <=
 // ||r|| + beta ||p_prev||) with its power-of-two FP16 scale
-__global__ void k_gram_scalars(CgArgs a, int it, float* beta, int* done, double* pn, float* pscale) {
-  const int b = blockIdx.x;
+// three warps, one sum each
+__global__ void __launch_bounds__(96) k_gram_scalars(CgArgs a, int it, float* beta, int* done, double* pn,
+                                                     float* pscale) {
+  __shared__ double sum[3];
+  const int b = blockIdx.x, w = threadIdx.x >> 5;
   const double* base = a.rr_part + (size_t)b * (a.itmax + 1) * a.PB;
-  const double rr = warp_sum_parts(base + (size_t)it * a.PB, a.PB);
-  const double rr0 = warp_sum_parts(base, a.PB);
-  const double rrp = it > 0 ? warp_sum_parts(base + (size_t)(it - 1) * a.PB, a.PB) : 1.0;
+  const int at = w == 0 ? it : w == 1 ? 0 : it - 1;
+  const double v = at >= 0 ? warp_sum_parts_long(base + (size_t)at * a.PB, a.PB) : 1.0;
+  if ((threadIdx.x & 31) == 0) sum[w] = v;
+  __syncthreads();
   if (threadIdx.x == 0) {
+    const double rr = sum[0], rr0 = sum[1], rrp = sum[2];
     done[b] = !(rr > a.rtol2 * rr0);
     const float bt = it > 0 ? (float)(rr / rrp) : 0.f;
     beta[b] = bt;
@@ -1221,7 +1226,7 @@ void launch_gram_build(const float2* smaps, const uint8_t* mask_host, int nc, co
 
 void launch_gram_scalars(const CgArgs& a, int nb, int it, float* beta, int* done, double* pn, float* pscale,
                          cudaStream_t s) {
-  k_gram_scalars<<<nb, 32, 0, s>>>(a, it, beta, done, pn, pscale);
+  k_gram_scalars<<<nb, 96, 0, s>>>(a, it, beta, done, pn, pscale);
 }
 
 void launch_gram_apply_scale(const float* x, int ny, int nx, int nb, float* pscale, cudaStream_t s) {
