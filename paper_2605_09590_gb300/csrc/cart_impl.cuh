@@ -70,6 +70,14 @@ struct NormShape {
   // then puts them on different bank halves (conflict-free), and the four
   // groups of a warp share a parity -- for uniform R = 2 masks also a mask class.
   static constexpr int KST = N1 * NC + ((N1 * NC) % 16 == 0 ? 4 : 12);
+  // Blocks per SM the kernel is compiled for: three, but two of 192 threads
+  // rather than three that spill 264 bytes a thread (384 x 384, 16 images,
+  // 8 coils, 10 CG iterations: 1448 -> 1240 us), and also four of 128 threads
+  // (128 registers, FOUR) for launches that three per SM do not hold at once:
+  // 256 x 256, 16 images (512 blocks) 732 -> 530 us, 48 images 1686 -> 1430 us.
+  // Launches that fit stay with three (2-3 % faster there).
+  static constexpr int MINB = N1 <= 20 ? 3 : 2;
+  static constexpr bool FOUR = NT == 128 && N2 == 16;
   static constexpr size_t buf = (size_t)N2 * KST * sizeof(float2);
   static constexpr size_t stile = (size_t)N * NC * sizeof(float2);
   static constexpr size_t smem = buf + 2 * stile + (size_t)N * sizeof(float2) + (size_t)N * sizeof(float) + 64;
@@ -88,8 +96,8 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src,
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-template <int N1, int N2, bool CG>
-__global__ void __launch_bounds__(NormShape<N1, N2>::NT, 3)
+template <int N1, int N2, bool CG, int MINB>
+__global__ void __launch_bounds__(NormShape<N1, N2>::NT, MINB)
     k_col_normal(CartOp op, const float2* __restrict__ xin, float2* __restrict__ yout, float lam, CgArgs a,
                  int it) {
   using Sh = NormShape<N1, N2>;
@@ -433,21 +441,28 @@ __global__ void __launch_bounds__(RowShape<M1, M2>::NT, (RowShape<M1, M2>::NT <=
 // ---------------------------------------------------------------------------
 // launchers (explicitly instantiated per size in the cart_inst_*.cu units)
 // ---------------------------------------------------------------------------
+template <int N1, int N2, int MINB>
+void launch_col_normal_m(const CartOp& op, const float2* x, float2* y, int nb, float lam, const CgArgs* a, int it,
+                         cudaStream_t s) {
+  using Sh = NormShape<N1, N2>;
+  const dim3 grid(cart_normal_tiles(op.nx), nb);
+  auto k = a ? k_col_normal<N1, N2, true, MINB> : k_col_normal<N1, N2, false, MINB>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem);
+  k<<<grid, Sh::NT, Sh::smem, s>>>(op, x, y, lam, a ? *a : CgArgs{}, it);
+}
+
 template <int N1, int N2>
 void launch_col_normal_t(const CartOp& op, const float2* x, float2* y, int nb, float lam, const CgArgs* a, int it,
                          cudaStream_t s) {
   using Sh = NormShape<N1, N2>;
-  const dim3 grid(cart_normal_tiles(op.nx), nb);
-  if (a) {
-    auto k = k_col_normal<N1, N2, true>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem);
-    k<<<grid, Sh::NT, Sh::smem, s>>>(op, nullptr, nullptr, lam, *a, it);
-  } else {
-    auto k = k_col_normal<N1, N2, false>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem);
-    CgArgs dummy{};
-    k<<<grid, Sh::NT, Sh::smem, s>>>(op, x, y, lam, dummy, 0);
+  if constexpr (Sh::FOUR) {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if ((int64_t)cart_normal_tiles(op.nx) * nb > (int64_t)Sh::MINB * nsm)
+      return launch_col_normal_m<N1, N2, Sh::MINB + 1>(op, x, y, nb, lam, a, it, s);
   }
+  launch_col_normal_m<N1, N2, Sh::MINB>(op, x, y, nb, lam, a, it, s);
 }
 
 template <int N1, int N2>

@@ -128,10 +128,9 @@ __device__ __forceinline__ void st_word(unsigned long long* p, unsigned seq, uns
   const unsigned long long w = ((unsigned long long)seq << 32) | payload;
   asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
 }
-__device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-  return w;
+// both words of an entry in one request (each on its own tells whether it is there)
+__device__ __forceinline__ void ld_words(const ulonglong2* p, unsigned long long& w0, unsigned long long& w1) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(w0), "=l"(w1) : "l"(p) : "memory");
 }
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
@@ -214,9 +213,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2)
         for (int m = 0; m < 4; ++m) {
           const int e = e0 + m, i = e / nj, jj = lane + 32 * (e % nj), b = b0 + warp + 8 * i;
           if (e < ne && jj < nx && b < nb) {
-            const ulonglong2* pe = part + (size_t)b * nx + jj;
-            w0[m] = ld_word(&pe->x);
-            w1[m] = ld_word(&pe->y);
+            ld_words(part + (size_t)b * nx + jj, w0[m], w1[m]);
           } else {
             w0[m] = w1[m] = (unsigned long long)seq << 32;
           }
@@ -535,14 +532,31 @@ bool launch_colcg_small(const float2* G, const float* gmax, const float2* rhs, f
                         int max_iter, double rtol2, float lam, double* rr0, double* rr, int* iters, int* status,
                         const SmallGlobal* glob, cudaStream_t s) {
   if (nb <= 0) return true;
-  // images per block: 32 for ny = 32, 16 for ny = 64 (128 blocks for 64
-  // columns and 32 images) and ny = 96 (shared memory)
-  if (ny == 32) return launch_small<32, 32>(G, gmax, rhs, X, nx, nb, max_iter, rtol2, lam, rr0, rr, iters, status, glob,
-                                    s);
-  if (ny == 64) return launch_small<64, 16>(G, gmax, rhs, X, nx, nb, max_iter, rtol2, lam, rr0, rr, iters, status, glob,
-                                    s);
-  if (ny == 96) return launch_small<96, 16>(G, gmax, rhs, X, nx, nb, max_iter, rtol2, lam, rr0, rr, iters, status, glob,
-                                    s);
+  // images per block: 32 for ny = 32, 16 for ny = 64 and 96 (shared memory); 16
+  // and 8 while the device then still takes every block at once, one per SM --
+  // the time is the latency of a block's updates, which the images of a block
+  // share (ny = 32, 64 columns, 32 images: 734 us with 32, 339 us with 16; 30
+  // iterations).  The bits do not depend on it.
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  auto fits = [&](int t) { return (int64_t)nx * ((nb + t - 1) / t) <= nsm; };
+#define PICO_SMALL(NY, T) \
+  return launch_small<NY, T>(G, gmax, rhs, X, nx, nb, max_iter, rtol2, lam, rr0, rr, iters, status, glob, s)
+  if (ny == 32) {
+    if (fits(8)) PICO_SMALL(32, 8);
+    if (fits(16)) PICO_SMALL(32, 16);
+    PICO_SMALL(32, 32);
+  }
+  if (ny == 64) {
+    if (fits(8)) PICO_SMALL(64, 8);
+    PICO_SMALL(64, 16);
+  }
+  if (ny == 96) {
+    if (fits(8)) PICO_SMALL(96, 8);
+    PICO_SMALL(96, 16);
+  }
+#undef PICO_SMALL
   return false;
 }
 
