@@ -216,6 +216,7 @@ bool launch_colcg_small(const float2* G, const float* gmax, const float2* rhs, f
 void launch_from_cp(const float* in, float2* out, int ny, int nx, int nb, cudaStream_t s);
 
 // ---- spiral.cu: non-Cartesian (Toeplitz normal operator, KB gridding) ----
+constexpr int kMaxTaps = 10;  // window integers for kb_width <= 8, plus one
 struct SpiralOp {
   int n;                    // image is n x n
   int L;                    // grid 2n

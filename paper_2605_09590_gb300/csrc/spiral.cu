@@ -12,6 +12,8 @@ bool launch_toep_normal_t(const SpiralOp&, const float2*, float2*, float2*, int,
 template <int P1, int P2>
 void launch_fft2_t(float2*, const float2*, int, int, bool, cudaStream_t);
 template <int P1, int P2>
+void launch_grid_rows_adjoint_t(const SpiralOp&, float2*, int, cudaStream_t);
+template <int P1, int P2>
 void launch_grid_cols_adjoint_t(const SpiralOp&, const float2*, float2*, int, cudaStream_t);
 
 namespace {
@@ -99,16 +101,21 @@ __global__ void k_toep_finalize(const float2* c, int64_t count, float scale, flo
 }
 
 // Gather-form Kaiser-Bessel gridding of PMR noise onto the 2n grid.
-// CTA: one 16x16 grid tile, one replica, kCoilGroup coils; thread = grid point.
+// CTA: one 16x16 grid tile, one replica, CG coils; thread = grid point.
 // The kernel is separable, phi(dx) phi(dy), and its 1-D weights at the integer
 // offsets of a sample's window (kMaxTaps of them, zero outside |d| <= W/2)
 // depend on the trajectory alone: k_grid_table evaluates them once per
 // sample at set-up.  Per staged chunk of a tile's samples the block copies
 // their weights and draws their noise (every thread one (sample, coil) pair),
 // then every grid point looks its two weights up -- no Bessel evaluation in
-// the gridding itself.
-constexpr int kCoilGroup = 4;
-constexpr int kMaxTaps = 10;  // window integers for kb_width <= 8, plus one
+// the gridding itself.  Most of a grid point's work is testing samples whose
+// window misses it (49 of a tile's 256 points are inside one), and that test is
+// the same for every coil: CG is as large as registers and shared memory allow,
+// up to 12.  32 replicas of 20 coils, 16384 samples on a 480 grid: 1609 us with 4
+// coils per block, 1040 us with 10, 910 us with the central tiles first, 818 us
+// with the warps' sample lists below.  What is left is the issue of the central
+// tiles (a spiral's four hold 2000-4000 samples each, the mean tile 40-80), one
+// block each: 6 images of 12 coils take 374 us, nearly all of it theirs.
 
 __global__ void k_grid_table(SpiralOp op, float* __restrict__ gw, int2* __restrict__ go) {
   const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -131,25 +138,32 @@ __global__ void k_grid_table(SpiralOp op, float* __restrict__ gw, int2* __restri
   go[m] = make_int2(((ix0 % L) + L) % L, ((iy0 % L) + L) % L);
 }
 
+template <int CG>
 __global__ void __launch_bounds__(256) k_grid_pmr(SpiralOp op, float2* __restrict__ Q, uint64_t seed,
                                                   int64_t rep_begin, float sigma, const float2* __restrict__ data) {
   __shared__ float s_wx[kChunk][kMaxTaps];
   __shared__ float s_wy[kChunk][kMaxTaps];
   __shared__ int2 s_o[kChunk];               // wrapped first grid index of each window (x, y)
   __shared__ int s_m[kChunk];                // sample index
-  __shared__ float2 s_w[kChunk][kCoilGroup];
+  __shared__ __align__(16) float2 s_w[kChunk][CG];
   const int L = op.L;
   const int tiles_x = L / 16;
-  const int tile = blockIdx.x;
-  const int b = blockIdx.y;
-  const int c0 = blockIdx.z * kCoilGroup;
-  const int ty = tile / tiles_x, tx = tile % tiles_x;
+  // replica and coil group vary fastest, tiles from the centre of k-space (index
+  // 0, wrapped) outwards: a spiral's central tiles hold many times the samples of
+  // the others and would otherwise run last, alone
+  const int groups = (op.nc + CG - 1) / CG;
+  const int b = blockIdx.x / groups;
+  const int c0 = (blockIdx.x % groups) * CG;
+  auto outwards = [&](int i) { return i & 1 ? tiles_x - (i + 1) / 2 : i / 2; };
+  const int ty = outwards(blockIdx.y / tiles_x), tx = outwards(blockIdx.y % tiles_x);
+  const int tile = ty * tiles_x + tx;
   const int gy = ty * 16 + threadIdx.x / 16, gx = tx * 16 + threadIdx.x % 16;
+  const int lane = threadIdx.x & 31;
   const uint64_t key = splitmix64(seed, (uint64_t)(rep_begin + b));
   const int beg = op.tile_ptr[tile], end = op.tile_ptr[tile + 1];
-  float2 acc[kCoilGroup];
+  float2 acc[CG];
 #pragma unroll
-  for (int g = 0; g < kCoilGroup; ++g) acc[g] = make_float2(0.f, 0.f);
+  for (int g = 0; g < CG; ++g) acc[g] = make_float2(0.f, 0.f);
   const float hw = op.halfw;
   const int ntaps = min(kMaxTaps, (int)(2.f * hw) + 2);
   for (int p0 = beg; p0 < end; p0 += kChunk) {
@@ -169,8 +183,8 @@ __global__ void __launch_bounds__(256) k_grid_pmr(SpiralOp op, float2* __restric
       else
         s_wy[i][k - kMaxTaps] = w;
     }
-    for (int j = threadIdx.x; j < cnt * kCoilGroup; j += blockDim.x) {
-      const int i = j / kCoilGroup, g = j - i * kCoilGroup;
+    for (int j = threadIdx.x; j < cnt * CG; j += blockDim.x) {
+      const int i = j / CG, g = j - i * CG;
       const int m = s_m[i], c = c0 + g;
       float2 v = make_float2(0.f, 0.f);
       if (c < op.nc) {
@@ -180,25 +194,51 @@ __global__ void __launch_bounds__(256) k_grid_pmr(SpiralOp op, float2* __restric
       s_w[i][g] = v;
     }
     __syncthreads();
-    for (int i = 0; i < cnt; ++i) {
-      const int2 o = s_o[i];
-      int kx = gx - o.x, ky = gy - o.y;
-      if (kx < 0) kx += L;
-      if (ky < 0) ky += L;
-      if (kx < ntaps && ky < ntaps) {
-        const float wgt = s_wx[i][kx] * s_wy[i][ky];
-        if (wgt != 0.f) {
+    // a warp owns two grid rows: its lanes test 32 samples at once against them, and
+    // the warp visits those whose window touches its points, in sample order
+    for (int i0 = 0; i0 < cnt; i0 += 32) {
+      bool near = false;
+      if (i0 + lane < cnt) {
+        const int2 o = s_o[i0 + lane];
+        int dx = tx * 16 - o.x, dy = gy - lane / 16 - o.y;
+        if (dx < 0) dx += L;
+        if (dy < 0) dy += L;
+        near = (dy < ntaps || dy == L - 1) && (dx < ntaps || dx >= L - 15);
+      }
+      // four at a time: their windows and weights are looked up together, or the
+      // look-ups of a dense tile's samples are one chain of latencies
+      for (unsigned todo = __ballot_sync(0xffffffffu, near); todo;) {
+        constexpr int U = 4;
+        int is[U];
+        float wgt[U];
 #pragma unroll
-          for (int g = 0; g < kCoilGroup; ++g) {
-            acc[g].x = fmaf(wgt, s_w[i][g].x, acc[g].x);
-            acc[g].y = fmaf(wgt, s_w[i][g].y, acc[g].y);
-          }
+        for (int u = 0; u < U; ++u) {
+          const bool on = todo != 0;
+          is[u] = on ? i0 + __ffs(todo) - 1 : i0;
+          todo &= todo - 1;
+          const int2 o = s_o[is[u]];
+          int kx = gx - o.x, ky = gy - o.y;
+          if (kx < 0) kx += L;
+          if (ky < 0) ky += L;
+          wgt[u] = on && kx < ntaps && ky < ntaps ? s_wx[is[u]][kx] * s_wy[is[u]][ky] : 0.f;
         }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (wgt[u] != 0.f) {
+#pragma unroll
+            for (int g = 0; g < CG; g += 2) {
+              const float4 v = *reinterpret_cast<const float4*>(&s_w[is[u]][g]);
+              acc[g].x = fmaf(wgt[u], v.x, acc[g].x);
+              acc[g].y = fmaf(wgt[u], v.y, acc[g].y);
+              acc[g + 1].x = fmaf(wgt[u], v.z, acc[g + 1].x);
+              acc[g + 1].y = fmaf(wgt[u], v.w, acc[g + 1].y);
+            }
+          }
       }
     }
   }
 #pragma unroll
-  for (int g = 0; g < kCoilGroup; ++g) {
+  for (int g = 0; g < CG; ++g) {
     const int c = c0 + g;
     if (c < op.nc) Q[(((size_t)b * op.nc + c) * L + gy) * L + gx] = acc[g];
   }
@@ -277,14 +317,24 @@ void launch_grid_table(const SpiralOp& op, float* gw, int2* go, cudaStream_t s) 
 void launch_grid_pmr(const SpiralOp& op, float2* Q, int nb, uint64_t seed, int64_t rep_begin, float sigma,
                      cudaStream_t s, const float2* data) {
   const int tiles = (op.L / 16) * (op.L / 16);
-  const dim3 grid(tiles, nb, (op.nc + kCoilGroup - 1) / kCoilGroup);
-  k_grid_pmr<<<grid, 256, 0, s>>>(op, Q, seed, rep_begin, sigma, data);
+  const int groups = (op.nc + 11) / 12, per = (op.nc + groups - 1) / groups;  // even groups of at most 12 coils
+  auto run = [&](auto kern, int cg) {
+    kern<<<dim3(nb * ((op.nc + cg - 1) / cg), tiles), 256, 0, s>>>(op, Q, seed, rep_begin, sigma, data);
+  };
+  if (per <= 4)
+    run(k_grid_pmr<4>, 4);
+  else if (per <= 8)
+    run(k_grid_pmr<8>, 8);
+  else if (per <= 10)
+    run(k_grid_pmr<10>, 10);
+  else
+    run(k_grid_pmr<12>, 12);
 }
 
 void launch_grid_adjoint_rest(const SpiralOp& op, float2* Q, float2* out, int nb, cudaStream_t s) {
 #define PICO_CASE(LL, A, B)                                        \
   if (op.P1 == A && op.P2 == B) {                                  \
-    launch_fft2_t<A, B>(Q, op.tw2, nb * op.nc, 1, true, s);        \
+    launch_grid_rows_adjoint_t<A, B>(op, Q, nb, s);                \
     launch_grid_cols_adjoint_t<A, B>(op, Q, out, nb, s);           \
     return;                                                        \
   }

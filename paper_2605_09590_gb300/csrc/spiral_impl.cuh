@@ -569,20 +569,70 @@ __global__ void __launch_bounds__(Split<P1, P2>::NT, 1) k_fft_cols(float2* __res
 }
 
 // ---------------------------------------------------------------------------
+// PMR adjoint, row pass: inverse row FFT of every grid row, in place; only the
+// columns that the centred crop keeps (N of L = 2N) are written.  Blocks of 128
+// threads on CS x kRowLines rows in the row passes' exchange layout, four per
+// SM, so that one block's loads and stores overlap another's transforms (640
+// planes of 480 x 480: one 480-thread block per SM and whole rows written 513 us,
+// now 395 us; 1.77 GB, two thirds of the HBM rate).
+// ---------------------------------------------------------------------------
+template <int P1, int P2>
+__global__ void __launch_bounds__(128, 4) k_grid_rows_adjoint(SpiralOp op, float2* __restrict__ data) {
+  using Rp = RowPass<P1, P2, 128>;
+  constexpr int L = P1 * P2, NT = 128, LINES = Rp::CS * Rp::RL, Q4 = L / 4;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  unsigned char* ex = smraw;
+  float2* twt = reinterpret_cast<float2*>(ex + LINES * Rp::line);  // [P2][P1]
+  const int t = threadIdx.x;
+  for (int i = t; i < L; i += NT) twt[i] = op.tw2[(i / P1) * (i % P1)];
+  __syncthreads();
+  float2* __restrict__ rows = data + (size_t)blockIdx.x * LINES * L;
+  for (int e = t; e < LINES * P1; e += NT) {
+    const int l = e / P1, n1 = e - l * P1;
+    float2 z[P2];
+#pragma unroll
+    for (int n2 = 0; n2 < P2; ++n2) z[n2] = rows[(size_t)l * L + n1 + P1 * n2];
+    DFT<P2, 1>::run(z);
+    unsigned char* x = ex + l * Rp::line;
+#pragma unroll
+    for (int k = 0; k < P2; k += 2) {
+      const float2 u = k == 0 ? z[0] : cmul_cb(z[k], twt[k * P1 + n1]), v = cmul_cb(z[k + 1], twt[(k + 1) * P1 + n1]);
+      *reinterpret_cast<float4*>(x + Rp::at(n1, k)) = make_float4(u.x, u.y, v.x, v.y);
+    }
+  }
+  __syncthreads();
+  const int l = t / P2, k2 = t % P2;
+  float2 y[P1];
+  const unsigned char* x = ex + l * Rp::line;
+#pragma unroll
+  for (int m = 0; m < P1; ++m) y[m] = *reinterpret_cast<const float2*>(x + Rp::at(m, k2));
+  DFT<P1, 1>::run(y);
+#pragma unroll
+  for (int k1 = 0; k1 < P1; ++k1) {
+    const int gx = k2 + P2 * k1;
+    if (gx < Q4 || gx >= L - Q4) rows[(size_t)l * L + gx] = y[k1];
+  }
+}
+
+// ---------------------------------------------------------------------------
 // PMR adjoint, last pass: inverse column FFT of the (row-transformed) grid,
 // centred crop to the N x N image, deapodisation and conj(S_c) coil combine.
 // Image column x reads grid column (x - N/2) mod L; image row y is grid row
-// (y - N/2) mod L.  One CTA: 16 image columns of one replica, all coils.
+// (y - N/2) mod L.  One CTA: 16 image columns of one replica, all coils; P2 x 16
+// threads, one b-job each, two blocks per SM or more.  Only the grid rows
+// k2 + P2 k1 with k1 in the first or last quarter can lie in the crop, so a
+// thread keeps 2 KA accumulators instead of P1 (32 replicas of 20 coils,
+// 240 x 240: one 480-thread block per SM, idle in the b-jobs, 661 us; now 199 us,
+// at the HBM rate of its 1.18 GB).
 // ---------------------------------------------------------------------------
 template <int P1, int P2>
-__global__ void __launch_bounds__(Split<P1, P2>::NT, 1)
+__global__ void __launch_bounds__(P2 * kLines, 512 / (P2 * kLines))
     k_grid_cols_adjoint(SpiralOp op, const float2* __restrict__ Q, float2* __restrict__ out) {
-  constexpr int L = P1 * P2;
-  constexpr int NT = Split<P1, P2>::NT;
+  constexpr int L = P1 * P2, NT = P2 * kLines, N = L / 2, KA = (P1 + 3) / 4;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* buf = reinterpret_cast<float2*>(smraw);
   float2* tws = buf + L * kLines;
-  const int t = threadIdx.x, N = op.n, b = blockIdx.y;
+  const int t = threadIdx.x, b = blockIdx.y;
   for (int i = t; i < L; i += NT) tws[i] = op.tw2[i];
   __syncthreads();
   const int ln = t % kLines, job = t / kLines;
@@ -590,40 +640,42 @@ __global__ void __launch_bounds__(Split<P1, P2>::NT, 1)
   const bool xval = x < N;
   const int gx = ((x - N / 2) % L + L) % L;
   const float dax = xval ? op.deapod[x] : 0.f;
-  float2 acc[P1];
+  float2 acc[2 * KA];
 #pragma unroll
-  for (int k1 = 0; k1 < P1; ++k1) acc[k1] = make_float2(0.f, 0.f);
+  for (int i = 0; i < 2 * KA; ++i) acc[i] = make_float2(0.f, 0.f);
   for (int c = 0; c < op.nc; ++c) {
     const float2* __restrict__ q = Q + ((size_t)b * op.nc + c) * L * L;
-    if (job < P1) {
+    for (int n1 = job; n1 < P1; n1 += P2) {
       float2 z[P2];
 #pragma unroll
-      for (int n2 = 0; n2 < P2; ++n2) z[n2] = xval ? q[(size_t)(job + P1 * n2) * L + gx] : make_float2(0.f, 0.f);
-      cola_store<P1, P2, 1>(z, job, ln, buf, tws);
+      for (int n2 = 0; n2 < P2; ++n2) z[n2] = xval ? q[(size_t)(n1 + P1 * n2) * L + gx] : make_float2(0.f, 0.f);
+      cola_store<P1, P2, 1>(z, n1, ln, buf, tws);
     }
     __syncthreads();
-    if (job < P2 && xval) {
+    if (xval) {
       float2 y[P1];
       colb_load<P1, P2>(y, job, ln, buf);
       DFT<P1, 1>::run(y);
 #pragma unroll
-      for (int k1 = 0; k1 < P1; ++k1) {
+      for (int i = 0; i < 2 * KA; ++i) {
+        const int k1 = i < KA ? i : P1 - 2 * KA + i;
         const int gy = job + P2 * k1;
         const int yy = (gy + N / 2) % L;  // image row of grid row gy
         if (yy < N) {
           const float2 s = __ldg(op.smaps + ((size_t)c * N + yy) * N + x);
-          acc[k1] = cfma_c(acc[k1], s, cscale(y[k1], dax * op.deapod[yy]));
+          acc[i] = cfma_c(acc[i], s, cscale(y[k1], dax * op.deapod[yy]));
         }
       }
     }
     __syncthreads();
   }
-  if (job < P2 && xval) {
+  if (xval) {
 #pragma unroll
-    for (int k1 = 0; k1 < P1; ++k1) {
+    for (int i = 0; i < 2 * KA; ++i) {
+      const int k1 = i < KA ? i : P1 - 2 * KA + i;
       const int gy = job + P2 * k1;
       const int yy = (gy + N / 2) % L;
-      if (yy < N) out[((size_t)b * N + yy) * N + x] = acc[k1];
+      if (yy < N) out[((size_t)b * N + yy) * N + x] = acc[i];
     }
   }
 }
@@ -727,13 +779,24 @@ void launch_fft2_t(float2* data, const float2* tw2, int planes, int sign, bool r
 }
 
 template <int P1, int P2>
+void launch_grid_rows_adjoint_t(const SpiralOp& op, float2* Q, int nb, cudaStream_t s) {
+  using Rp = RowPass<P1, P2, 128>;
+  constexpr int lines = Rp::CS * Rp::RL;   // divides L, a multiple of 16
+  const size_t sm = (size_t)lines * Rp::line + Rp::tw;
+  auto k = k_grid_rows_adjoint<P1, P2>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const int64_t blocks = (int64_t)nb * op.nc * (P1 * P2 / lines);
+  k<<<(unsigned)blocks, 128, sm, s>>>(op, Q);
+}
+
+template <int P1, int P2>
 void launch_grid_cols_adjoint_t(const SpiralOp& op, const float2* Q, float2* out, int nb, cudaStream_t s) {
   using Sp = Split<P1, P2>;
   constexpr int L = P1 * P2;
   const size_t sm = Sp::col_buf + L * sizeof(float2);
   auto k = k_grid_cols_adjoint<P1, P2>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k<<<dim3((op.n + kLines - 1) / kLines, nb), Sp::NT, sm, s>>>(op, Q, out);
+  k<<<dim3((op.n + kLines - 1) / kLines, nb), P2 * kLines, sm, s>>>(op, Q, out);
 }
 
 }  // namespace pico
