@@ -220,6 +220,7 @@ __global__ void k_axpy_bcast(float2* __restrict__ x, const float2* __restrict__ 
 constexpr int kTapMax = 8;
 constexpr int kFuseTX = 32;        // coefficients per tile and band along x
 constexpr int kFuseThreads = 256;
+constexpr int kLoadAhead = 6;      // global loads in flight per thread and operand
 
 struct FwdArgs {
   int n, m;                        // image side, side of this level's input region
@@ -239,19 +240,19 @@ enum { kLoadGrad, kLoadVjp, kLoadPlain };
 // kLoadVjp:   z = a - b s0 (0 if !a);  c' = a ? -s2 c : c;  c' + s1 z
 //             (reverse sweep: zb = yb - M yb / Lc, xk = xb + (1 + c_k) zb with xb = -c_{k+1} zb_prev)
 template <int LOAD>
-__device__ __forceinline__ float2 cs_load(const FwdArgs& f, size_t o, size_t i, int b, bool own) {
+__device__ __forceinline__ float2 cs_load(const FwdArgs& f, size_t o, size_t i, int b, float2& z) {
   if (LOAD == kLoadPlain) return f.a[o];
   if (LOAD == kLoadGrad) {
-    const float2 z = f.a[o], mz = f.b[o], r = f.c[(size_t)b * f.c_stride + i];
-    return make_float2(fmaf(-f.s0, mz.x - r.x, z.x), fmaf(-f.s0, mz.y - r.y, z.y));
+    const float2 zz = f.a[o], mz = f.b[o], r = f.c[(size_t)b * f.c_stride + i];
+    return make_float2(fmaf(-f.s0, mz.x - r.x, zz.x), fmaf(-f.s0, mz.y - r.y, zz.y));
   }
-  float2 z = make_float2(0.f, 0.f), xb = f.c[o];
+  float2 xb = f.c[o];
+  z = make_float2(0.f, 0.f);
   if (f.a) {
     const float2 y = f.a[o], my = f.b[o];
     z = make_float2(fmaf(-f.s0, my.x, y.x), fmaf(-f.s0, my.y, y.y));
     xb = make_float2(-f.s2 * xb.x, -f.s2 * xb.y);
   }
-  if (own) f.zout[o] = z;
   return make_float2(fmaf(f.s1, z.x, xb.x), fmaf(f.s1, z.y, xb.y));
 }
 
@@ -271,17 +272,30 @@ __global__ void __launch_bounds__(kFuseThreads) k_cs_fwd(FwdArgs f, Wavelet w) {
   const int t = threadIdx.x, b = blockIdx.z, n = f.n, m = f.m, half = m / 2;
   const int kx0 = blockIdx.x * TX, ky0 = blockIdx.y * TY;
   const size_t img = (size_t)b * n * n;
-  for (int e = t; e < IY * IX; e += kFuseThreads) {
-    const int r = e / IX, q = e - r * IX;
-    int y = 2 * ky0 + r, x = 2 * kx0 + q;
-    const bool own = r < 2 * TY && q < 2 * TX && y < m && x < m;
-    // the last tile's overhang beyond the periodic halo is loaded from a valid place and not used
-    if (y >= m) y -= m;
-    if (x >= m) x -= m;
-    y = min(y, m - 1);
-    x = min(x, m - 1);
-    const size_t i = (size_t)y * n + x;
-    in[r][q] = cs_load<LOAD>(f, img + i, i, b, own);
+  // kLoadAhead values per thread are requested before the first is used: the
+  // loads, not the transforms, are the time of a launch of few tiles
+  for (int e0 = t; e0 < IY * IX; e0 += kLoadAhead * kFuseThreads) {
+    float2 v[kLoadAhead], z[kLoadAhead];
+#pragma unroll
+    for (int u = 0; u < kLoadAhead; ++u) {
+      const int e = min(e0 + u * kFuseThreads, IY * IX - 1), r = e / IX, q = e - r * IX;
+      // the last tile's overhang beyond the periodic halo is loaded from a valid place and not used
+      int y = 2 * ky0 + r, x = 2 * kx0 + q;
+      if (y >= m) y -= m;
+      if (x >= m) x -= m;
+      const size_t i = (size_t)min(y, m - 1) * n + min(x, m - 1);
+      v[u] = cs_load<LOAD>(f, img + i, i, b, z[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kLoadAhead; ++u) {
+      const int e = e0 + u * kFuseThreads, r = e / IX, q = e - r * IX;
+      if (e >= IY * IX) break;
+      in[r][q] = v[u];
+      if (LOAD == kLoadVjp) {
+        const int y = 2 * ky0 + r, x = 2 * kx0 + q;
+        if (r < 2 * TY && q < 2 * TX && y < m && x < m) f.zout[img + (size_t)y * n + x] = z[u];
+      }
+    }
   }
   __syncthreads();
   for (int e = t; e < IY * TX; e += kFuseThreads) {
@@ -353,14 +367,22 @@ __global__ void __launch_bounds__(kFuseThreads) k_cs_inv(InvArgs f, Wavelet w) {
   const int t = threadIdx.x, b = blockIdx.z, n = f.n, m = f.m, half = m / 2;
   const int kx0 = blockIdx.x * TX, ky0 = blockIdx.y * TY;   // first own coefficient of the tile
   const size_t img = (size_t)b * n * n;
-  for (int e = t; e < 2 * CY * 2 * CX; e += kFuseThreads) {
-    const int hy = e / (CY * 2 * CX), r = (e / (2 * CX)) % CY, q = e % (2 * CX), hx = q >= CX;
-    int ky = ky0 + r - HB, kx = kx0 + (q - hx * CX) - HB;
-    if (ky < 0) ky += half;
-    if (kx < 0) kx += half;
-    ky = min(ky, half - 1);
-    kx = min(kx, half - 1);
-    in[hy][r][q] = f.src[img + (size_t)(ky + hy * half) * n + kx + hx * half];
+  for (int e0 = t; e0 < 2 * CY * 2 * CX; e0 += kLoadAhead * kFuseThreads) {
+    float2 v[kLoadAhead];
+#pragma unroll
+    for (int u = 0; u < kLoadAhead; ++u) {
+      const int e = min(e0 + u * kFuseThreads, 2 * CY * 2 * CX - 1);
+      const int hy = e / (CY * 2 * CX), r = (e / (2 * CX)) % CY, q = e % (2 * CX), hx = q >= CX;
+      int ky = ky0 + r - HB, kx = kx0 + (q - hx * CX) - HB;
+      if (ky < 0) ky += half;
+      if (kx < 0) kx += half;
+      v[u] = f.src[img + (size_t)(min(ky, half - 1) + hy * half) * n + min(kx, half - 1) + hx * half];
+    }
+#pragma unroll
+    for (int u = 0; u < kLoadAhead; ++u) {
+      const int e = e0 + u * kFuseThreads;
+      if (e < 2 * CY * 2 * CX) (&in[0][0][0])[e] = v[u];
+    }
   }
   __syncthreads();
   for (int e = t; e < 2 * TY * 2 * CX; e += kFuseThreads) {
@@ -442,7 +464,18 @@ __global__ void __launch_bounds__(kCoreThreads) k_cs_core(float2* data, int n, i
   float2 *A = core, *B = core + m * m;
   float2* img = data + (size_t)blockIdx.x * n * n;
   const int t = threadIdx.x;
-  for (int e = t; e < m * m; e += kCoreThreads) A[e] = img[(size_t)(e / m) * n + e % m];
+  constexpr int U = kCoreSide * kCoreSide / kCoreThreads;   // values per thread
+  {
+    float2 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = min(t + u * kCoreThreads, m * m - 1);
+      v[u] = img[(size_t)(e / m) * n + e % m];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (t + u * kCoreThreads < m * m) A[t + u * kCoreThreads] = v[u];
+  }
   __syncthreads();
   for (int l = 0; l < levels; ++l) {
     const int s = m >> l, half = s / 2;
@@ -457,9 +490,10 @@ __global__ void __launch_bounds__(kCoreThreads) k_cs_core(float2* data, int n, i
     }
     __syncthreads();
   }
-  for (int e = t; e < m * m; e += kCoreThreads) {
-    const size_t i = (size_t)(e / m) * n + e % m;
-    A[e] = cs_threshold<TAN>(A[e], i, at, keep, tau);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int e = t + u * kCoreThreads;
+    if (e < m * m) A[e] = cs_threshold<TAN>(A[e], (size_t)(e / m) * n + e % m, at, keep, tau);
   }
   __syncthreads();
   for (int l = levels - 1; l >= 0; --l) {
