@@ -902,7 +902,7 @@ void noise_adjoint(pico_ctx* c, float2* out, int nb, uint64_t seed, int64_t rep_
     adjoint2d_from_kbuf(c, out, nb);
   } else if (c->kind == PICO_CARTESIAN) {
     { Launch L(c, 2); pico::launch_cart_pmr_cols(c->cop, c->G, nb, seed, rep_begin, (float)sigma, c->stream); }
-    { Launch L(c, 2); pico::launch_cart_rows_adjoint(c->cop, c->G, out, nb, c->stream); }
+    { Launch L(c, 2); pico::launch_cart_rows_adjoint(c->cop, c->G, out, nb, c->g_err, c->stream); }
   } else {
     { Launch L(c, 2); pico::launch_grid_pmr(c->sop, c->G, nb, seed, rep_begin, (float)sigma, c->stream); }
     { Launch L(c, 2, 2); pico::launch_grid_adjoint_rest(c->sop, c->G, out, nb, c->stream); }
@@ -1522,7 +1522,8 @@ pico_status pico_adjoint(pico_ctx* c, const void* y, void* x, int32_t nbatch) {
       adjoint2d_from_kbuf(c, xo + (size_t)b0 * c->n, nb);
     } else if (c->kind == PICO_CARTESIAN) {
       { Launch L(c, 3); pico::launch_cart_pmr_cols(c->cop, c->G, nb, 0, 0, 0.f, c->stream, yb); }
-      { Launch L(c, 3); pico::launch_cart_rows_adjoint(c->cop, c->G, xo + (size_t)b0 * c->n, nb, c->stream); }
+      { Launch L(c, 3); pico::launch_cart_rows_adjoint(c->cop, c->G, xo + (size_t)b0 * c->n, nb, c->g_err,
+                                                              c->stream); }
     } else {
       { Launch L(c, 3); pico::launch_grid_pmr(c->sop, c->G, nb, 0, 0, 0.f, c->stream, yb); }
       { Launch L(c, 3, 2); pico::launch_grid_adjoint_rest(c->sop, c->G, xo + (size_t)b0 * c->n, nb, c->stream); }

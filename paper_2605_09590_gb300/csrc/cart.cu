@@ -9,7 +9,7 @@ void launch_col_normal_t(const CartOp&, const float2*, float2*, int, float, cons
 template <int N1, int N2>
 void launch_col_pmr_t(const CartOp&, float2*, int, uint64_t, int64_t, float, cudaStream_t, const float2*);
 template <int M1, int M2>
-void launch_row_adjoint_t(const CartOp&, const float2*, float2*, int, cudaStream_t);
+void launch_row_adjoint_t(const CartOp&, const float2*, float2*, int, int*, cudaStream_t);
 
 static bool split_of(int n, int* a, int* b) {
 #define PICO_SPLIT(N, A, B) \
@@ -53,9 +53,9 @@ void launch_cart_pmr_cols(const CartOp& op, float2* G, int nb, uint64_t seed, in
 #undef PICO_CASE
 }
 
-void launch_cart_rows_adjoint(const CartOp& op, const float2* G, float2* out, int nb, cudaStream_t s) {
+void launch_cart_rows_adjoint(const CartOp& op, const float2* G, float2* out, int nb, int* err, cudaStream_t s) {
 #define PICO_CASE(N, A, B) \
-  if (op.M1 == A && op.M2 == B) return launch_row_adjoint_t<A, B>(op, G, out, nb, s);
+  if (op.M1 == A && op.M2 == B) return launch_row_adjoint_t<A, B>(op, G, out, nb, err, s);
   PICO_SIZES(PICO_CASE)
 #undef PICO_CASE
 }

@@ -19,6 +19,8 @@
 #include "common.cuh"
 #include "dft_codelets.cuh"
 #include "kernels.cuh"
+#include "row_pass.cuh"
+#include "tc_util.cuh"
 
 namespace pico {
 
@@ -438,6 +440,104 @@ __global__ void __launch_bounds__(RowShape<M1, M2>::NT, (RowShape<M1, M2>::NT <=
   }
 }
 
+// The same with blocks of four rows that take several coils per step (RowPass:
+// one coil per a-thread and group of CS): hybrid rows arrive by TMA tensor loads
+// in the swizzled exchange layout, sensitivity rows by bulk copies, both while
+// other work runs, and four blocks share an SM.  256 replicas of 15 coils at
+// 320 x 320: k_row_adjoint (16 rows, two 320-thread blocks per SM, strided
+// twiddle look-ups) 1042 us, this 922 us; the hybrid's 3.15 GB take 464 us.
+template <int M1, int M2, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT)
+    k_row_adjoint_v(CartOp op, const __grid_constant__ CUtensorMap mG, float2* __restrict__ out, int* err) {
+  using Rp = RowPass<M1, M2, NT>;
+  constexpr int RL = Rp::RL, CS = Rp::CS, M = M1 * M2;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  unsigned char* ex = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
+  float2* sst = reinterpret_cast<float2*>(ex + CS * Rp::slot);  // [CS][RL][M]
+  float2* twt = sst + CS * RL * M;                              // [M2][M1]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(twt + M);
+  const int t = threadIdx.x, b = blockIdx.y, y0 = blockIdx.x * RL, ny = op.ny;
+  if (t == 0) {
+    tc::mbar_init(bar, 1);
+    tc::mbar_init(bar + 1, 1);
+    tc::fence_mbar_init();
+  }
+  for (int i = t; i < M; i += NT) twt[i] = op.twx[(i / M1) * (i % M1)];
+  __syncthreads();
+  auto issue_g = [&](int c0) {
+    const int cn = min(CS, op.nc - c0);
+    tc::mbar_expect_tx(bar, (uint32_t)(cn * RL * M * 8));
+    for (int l = 0; l < cn * RL; ++l)
+      tc::tma_load_3d(ex + l * Rp::line, &mG, bar, 0, 0, (b * op.nc + c0 + l / RL) * ny + y0 + l % RL);
+  };
+  auto issue_s = [&](int c0) {
+    const int cn = min(CS, op.nc - c0);
+    tc::mbar_expect_tx(bar + 1, (uint32_t)(cn * RL * M * 8));
+    for (int c = 0; c < cn; ++c)
+      tc::bulk_load(sst + c * RL * M, op.smaps + ((size_t)(c0 + c) * ny + y0) * M, RL * M * 8, bar + 1);
+  };
+  if (t == 0) issue_g(0);
+  const int ra = t / M1, n1 = t - ra * M1;
+  const bool ajob = t < RL * M1;
+  const int cb = t / (RL * M2), rb = (t / M2) % RL, k2 = t % M2;
+  float2 acc[M2];
+#pragma unroll
+  for (int n2 = 0; n2 < M2; ++n2) acc[n2] = make_float2(0.f, 0.f);
+  bool ok = true;
+  int phase = 0;
+  for (int c0 = 0; c0 < op.nc; c0 += CS, phase ^= 1) {
+    if (ok && !tc::mbar_wait(bar, phase)) {  // reported by pico_sync; the block runs on so that its barriers pair up
+      ok = false;
+      if (err) atomicCAS(err, 0, 13);
+    }
+    if (c0 + cb < op.nc) {
+      float2 y[M1];
+      unsigned char* e = ex + cb * Rp::slot + rb * Rp::line;
+#pragma unroll
+      for (int m = 0; m < M1; ++m) y[m] = *reinterpret_cast<const float2*>(e + Rp::at(m, k2));
+      DFT<M1, 1>::run(y);
+#pragma unroll
+      for (int m = 0; m < M1; ++m) *reinterpret_cast<float2*>(e + Rp::at(m, k2)) = y[m];
+    }
+    __syncthreads();  // rows transformed; the sensitivities of the step before were last read before it
+    if (t == 0) issue_s(c0);
+#pragma unroll 1
+    for (int j = 0; j < CS; ++j) {
+      const bool on = ajob && c0 + j < op.nc;
+      const unsigned char* e = ex + j * Rp::slot + ra * Rp::line;
+      float2 z[M2];
+      if (on) {
+#pragma unroll
+        for (int k = 0; k < M2; k += 2) {
+          const float4 v = *reinterpret_cast<const float4*>(e + Rp::at(n1, k));
+          z[k] = k == 0 ? make_float2(v.x, v.y) : cmul_cb(make_float2(v.x, v.y), twt[k * M1 + n1]);
+          z[k + 1] = cmul_cb(make_float2(v.z, v.w), twt[(k + 1) * M1 + n1]);
+        }
+      }
+      if (j == CS - 1) {
+        tc::fence_proxy_async_smem();  // the in-place writes before the next step's copies
+        __syncthreads();               // the slots are free
+        if (t == 0 && c0 + CS < op.nc) issue_g(c0 + CS);
+      }
+      if (on) DFT<M2, 1>::run(z);
+      if (j == 0 && ok && !tc::mbar_wait(bar + 1, phase)) {
+        ok = false;
+        if (err) atomicCAS(err, 0, 13);
+      }
+      if (on) {
+        const float2* S = sst + (j * RL + ra) * M + n1;
+#pragma unroll
+        for (int n2 = 0; n2 < M2; ++n2) acc[n2] = cfma_c(acc[n2], S[M1 * n2], z[n2]);
+      }
+    }
+  }
+  if (ajob) {
+    float2* __restrict__ o = out + ((size_t)b * ny + y0 + ra) * M + n1;
+#pragma unroll
+    for (int n2 = 0; n2 < M2; ++n2) o[M1 * n2] = acc[n2];
+  }
+}
+
 // ---------------------------------------------------------------------------
 // launchers (explicitly instantiated per size in the cart_inst_*.cu units)
 // ---------------------------------------------------------------------------
@@ -477,7 +577,24 @@ void launch_col_pmr_t(const CartOp& op, float2* G, int nb, uint64_t seed, int64_
 }
 
 template <int M1, int M2>
-void launch_row_adjoint_t(const CartOp& op, const float2* G, float2* out, int nb, cudaStream_t s) {
+void launch_row_adjoint_t(const CartOp& op, const float2* G, float2* out, int nb, int* err, cudaStream_t s) {
+  if constexpr (M2 >= 8) {
+    // four-row blocks once they fill the device (two per SM); few of them are
+    // quicker as blocks of 16 rows and 16 M1 threads
+    constexpr int NT = kRowLines * M1 <= 64 ? 64 : 128;
+    using Rp = RowPass<M1, M2, NT>;
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    CUtensorMap mG{};
+    if (op.ny % kRowLines == 0 && (int64_t)nb * (op.ny / kRowLines) > 2 * nsm &&
+        encode_row_map(&mG, G, M1, M2, (int64_t)nb * op.nc * op.ny, 1)) {
+      const size_t sm = Rp::smem(op.nx);
+      auto k = k_row_adjoint_v<M1, M2, NT>;
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      return k<<<dim3(op.ny / kRowLines, nb), NT, sm, s>>>(op, mG, out, err);
+    }
+  }
   using Sh = RowShape<M1, M2>;
   const dim3 grid((op.ny + kRowTile - 1) / kRowTile, nb);
   auto k = k_row_adjoint<M1, M2>;

@@ -97,7 +97,8 @@ void launch_cart_cg_normal(const CartOp& op, const CgArgs& a, int nb, int it, fl
 void launch_cart_pmr_cols(const CartOp& op, float2* G, int nb, uint64_t seed, int64_t rep_begin, float sigma,
                           cudaStream_t s, const float2* data = nullptr);
 // out[b] = sum_c conj(S_c) . F^H_x G[b][c]
-void launch_cart_rows_adjoint(const CartOp& op, const float2* G, float2* out, int nb, cudaStream_t s);
+// err: first failure code of a bounded wait (device)
+void launch_cart_rows_adjoint(const CartOp& op, const float2* G, float2* out, int nb, int* err, cudaStream_t s);
 
 // ---- gram.cu: dense per-column normal operator on the tensor cores ----
 struct GramOp {
