@@ -162,12 +162,12 @@ def kernel_digest(*names):
 GRAM_FILES = ("gram.cu", "tc_util.cuh", "kernels.cuh", "f16_split.cuh")
 PERSIST_FILES = ("colcg_persist.cu", "tc_util.cuh", "kernels.cuh", "f16_split.cuh")
 TRAFFIC = {
-    ("knee320_r2", 256, "gram", "580cead29cb443a1"): (713.137664e6 + 378.007808e6 + 711.760128e6 + 374.798592e6) / 2,
-    ("knee320_r2", 256, "persist", "b7cf5961e2e5f7f1"): (473.558528e6 + 375.167488e6 + 473.355264e6 + 371.994624e6) / 2,
+    ("knee320_r2", 256, "gram", "1d01b2522f49a155"): (714.505728e6 + 378.052864e6 + 713.128192e6 + 375.682560e6) / 2,
+    ("knee320_r2", 256, "persist", "a0617cf5af7283d1"): (473.113856e6 + 375.561728e6 + 473.358336e6 + 373.248256e6) / 2,
     # one spiral normal operator = k_toep_rows_fwd + k_toep_cols_w + k_toep_rows_inv (two of each averaged)
-    ("spiral240_r2", 256, "fft", "40fe3b9a9e3fec65"): ((4720.102912e6 + 4661.500160e6 + 4719.623168e6 + 4658.126080e6)
-                                                       + (5086.091520e6 + 133.305856e6 + 5086.246656e6 + 133.519616e6)
-                                                       + (474.891264e6 + 4772.518912e6 + 474.142464e6 + 4772.286208e6)) / 2,
+    ("spiral240_r2", 256, "fft", "d815e6bb16f247fe"): ((4721.042688e6 + 4658.534400e6 + 4720.445952e6 + 4655.390720e6)
+                                                       + (5019.997184e6 + 170.031360e6 + 5020.940544e6 + 170.595072e6)
+                                                       + (422.909952e6 + 4771.781120e6 + 421.893632e6 + 4771.749888e6)) / 2,
 }
 
 
@@ -219,7 +219,7 @@ def fft_roofline(w, K, avg_s, launches):
     flops = K * flops_per_probe(w)
     achieved = flops / avg_s / 1e12
     peak = N_SM * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
-    files = ("cart_impl.cuh", "kernels.cuh") if w.kind == "cartesian" else ("spiral_impl.cuh", "kernels.cuh")
+    files = ("cart_impl.cuh", "kernels.cuh") if w.kind == "cartesian" else ("spiral_impl.cuh", "row_pass.cuh", "kernels.cuh")
     traffic, dig = traffic_of(w, K, "fft", files)
     alg = alg_bytes_normal(w, K)
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
@@ -1031,7 +1031,7 @@ def bench_cs(args, w, inp, pico, torch, dist, world, rank, local, steps, warmup,
     hbm = images * (2 * img + 4 * w.nc * img) / (norm_ms / 1e3) / 1e9
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": None,
-            "kernel": "k_toep_rows_fwd + k_toep_cols + k_toep_rows_inv (2-D-mask normal operator, no padding)",
+            "kernel": "k_toep_rows_fwd + k_toep_cols_w + k_toep_rows_inv (2-D-mask normal operator, no padding)",
             "avg_launch_ms": avg_norm_s * 1e3, "launches": norm_n, "images": images,
             "peak_note": "FP32 FMA peak 152 SM x 128 lanes x 2 x 2070 MHz (nominal max clock); achieved = "
                          "algorithmic flops of every image through the operator / its total time",

@@ -1079,7 +1079,7 @@ pico_status init_impl(const pico_operator_desc* d, void* cuda_stream, size_t hbm
     if (c->ny != c->nx) return fail(c, PICO_E_UNSUPPORTED, "2-D masks need square images");
     if (!pico::grid_split(img, &P1, &P2) || !pico::fft_length_supported(img))
       return fail(c, PICO_E_UNSUPPORTED, "image size has no 2-D FFT split in this build");
-    PA = img / pico::kRowLines;
+    PA = (img + pico::kRowLines - 1) / pico::kRowLines;
     extra = std::max((size_t)B * nc * n, (size_t)n) * 8 + (size_t)n * 5 + (size_t)img * 8;
   } else if (c->kind == PICO_CARTESIAN) {
     if (!pico::cart_supported(c->ny, c->nx, &N1, &N2, &M1, &M2))
@@ -1099,7 +1099,7 @@ pico_status init_impl(const pico_operator_desc* d, void* cuda_stream, size_t hbm
     if (kbw < 2 || kbw > 8 || (kbw & 1)) return fail(c, PICO_E_UNSUPPORTED, "kb_width must be 2, 4, 6 or 8");
     if (!pico::spiral_supported(img, &P1, &P2))
       return fail(c, PICO_E_UNSUPPORTED, "spiral image size has no 2N grid split in this build");
-    PA = img / pico::kRowLines;
+    PA = (img + pico::kRowLines - 1) / pico::kRowLines;
     c->nsamp = d->nsamp;
     extra = std::max((size_t)B * nc * img * L, (size_t)L * L) * 8 + (size_t)L * L * 4 + (size_t)img * 4 + (size_t)L * 8 +
             (size_t)c->nsamp * (8 + 8 + 8 + 16 + 88) + (size_t)(L / 16) * (L / 16) * 4 + 64;
@@ -1242,7 +1242,7 @@ size_t footprint_bytes(const pico_operator_desc* d, bool with_kbuf) {
   const int64_t PB = (n + kVecPerBlock - 1) / kVecPerBlock;
   int64_t PA, extra, kbuf;
   if (d->kind == PICO_CARTESIAN && d->mask_2d) {
-    PA = d->ny / kRowLines;
+    PA = (d->ny + kRowLines - 1) / kRowLines;
     extra = std::max(B * nc * n, n) * 8 + n * 5 + (int64_t)d->ny * 8;
     kbuf = B * nc * n * 8;
   } else if (d->kind == PICO_CARTESIAN) {
@@ -1256,7 +1256,7 @@ size_t footprint_bytes(const pico_operator_desc* d, bool with_kbuf) {
     }
   } else {
     const int64_t img = d->ny, L = 2 * img;
-    PA = img / kRowLines;
+    PA = (img + kRowLines - 1) / kRowLines;
     extra = std::max(B * nc * img * L, L * L) * 8 + L * L * 4 + img * 4 + L * 8 + d->nsamp * (56 + 88) +
             (L / 16) * (L / 16) * 4 + 64;
     kbuf = B * nc * 4 * n * 8;
