@@ -165,9 +165,9 @@ TRAFFIC = {
     ("knee320_r2", 256, "gram", "1d01b2522f49a155"): (714.505728e6 + 378.052864e6 + 713.128192e6 + 375.682560e6) / 2,
     ("knee320_r2", 256, "persist", "a0617cf5af7283d1"): (473.113856e6 + 375.561728e6 + 473.358336e6 + 373.248256e6) / 2,
     # one spiral normal operator = k_toep_rows_fwd + k_toep_cols_w + k_toep_rows_inv (two of each averaged)
-    ("spiral240_r2", 256, "fft", "d815e6bb16f247fe"): ((4721.042688e6 + 4658.534400e6 + 4720.445952e6 + 4655.390720e6)
-                                                       + (5019.997184e6 + 170.031360e6 + 5020.940544e6 + 170.595072e6)
-                                                       + (422.909952e6 + 4771.781120e6 + 421.893632e6 + 4771.749888e6)) / 2,
+    ("spiral240_r2", 256, "fft", "188d8e988e3ab7fe"): ((4720.863488e6 + 4658.663168e6 + 4720.915712e6 + 4655.494144e6)
+                                                       + (5021.168128e6 + 170.465792e6 + 5022.122240e6 + 170.078208e6)
+                                                       + (418.384384e6 + 4771.740160e6 + 415.642368e6 + 4772.048896e6)) / 2,
 }
 
 

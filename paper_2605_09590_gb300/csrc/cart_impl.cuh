@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       for (int m = 0; m < M1; ++m) *reinterpret_cast<float2*>(e + Rp::at(m, k2)) = y[m];
     }
     __syncthreads();  // rows transformed; the sensitivities of the step before were last read before it
-    if (t == 0) issue_s(c0);
+    if (t == 0 && ok) issue_s(c0);
 #pragma unroll 1
     for (int j = 0; j < CS; ++j) {
       const bool on = ajob && c0 + j < op.nc;
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       if (j == CS - 1) {
         tc::fence_proxy_async_smem();  // the in-place writes before the next step's copies
         __syncthreads();               // the slots are free
-        if (t == 0 && c0 + CS < op.nc) issue_g(c0 + CS);
+        if (t == 0 && ok && c0 + CS < op.nc) issue_g(c0 + CS);
       }
       if (on) DFT<M2, 1>::run(z);
       if (j == 0 && ok && !tc::mbar_wait(bar + 1, phase)) {
@@ -531,6 +531,10 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       }
     }
   }
+  // after a time-out nothing more was requested: wait (bounded) for what was; of
+  // each barrier's two parities the completed one returns at once
+  if (t == 0 && !ok)
+    for (int i = 0; i < 4; ++i) tc::mbar_wait(bar + i / 2, i & 1, 200000000ull);
   if (ajob) {
     float2* __restrict__ o = out + ((size_t)b * ny + y0 + ra) * M + n1;
 #pragma unroll

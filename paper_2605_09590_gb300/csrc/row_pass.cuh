@@ -15,8 +15,8 @@ namespace pico {
 // Before, a block's one coil at a time left half of its threads without a b-job,
 // the strided twiddle look-ups made up most of the shared-memory wavefronts, and
 // every coil waited for its own global loads (ncu: issue 30-36 %, barrier and
-// load stalls 6 of 8 warps): 32 images at L = 480, forward 176 -> 132 us,
-// inverse 221 -> 157 us, now at 55 % of the DRAM rate.
+// load stalls 6 of 8 warps): 32 images at L = 480, forward 176 -> 138 us,
+// inverse 221 -> 171 us, now at half of the DRAM rate.
 //
 // Exchange layout: a line of each (coil, image row) holds P1 rows of P2 values,
 // row n1 the P2 values of that n1, with the 16-byte chunk of value k at

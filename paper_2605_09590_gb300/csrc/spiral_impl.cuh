@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       }
     }
     __syncthreads();  // exchange slots full, sensitivities read
-    if (t == 0 && c0 + CS < op.nc) issue(c0 + CS);
+    if (t == 0 && ok && c0 + CS < op.nc) issue(c0 + CS);
     if (c0 + cb < op.nc) {
       float2 y[P1];
       const unsigned char* e = ex + cb * Rp::slot + rb * Rp::line;
@@ -160,6 +160,8 @@ __global__ void __launch_bounds__(NT, 512 / NT)
     }
     __syncthreads();  // the slots are rewritten by the next step
   }
+  if (t == 0 && !ok)  // nothing more was requested: wait (bounded) for what was
+    for (int i = 0; i < 2; ++i) tc::mbar_wait(bar, i, 200000000ull);
 }
 
 // ---------------------------------------------------------------------------
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
 // the a-jobs in both directions (single look-ups W^(n1 k) by a- and b-jobs:
 // 2084 us against 2045 us, with the row passes below in place).
 // Bound by shared-memory wavefronts and the FP32 pipes at about half each (ncu,
-// 32 images: 56 % and 50 %): every value crosses shared memory five times, and
+// 32 images: 59 % and 47 %): every value crosses shared memory five times, and
 // two blocks of 8 warps overlap the two pipes only partly.
 template <int P1, int P2>
 struct ColsW {
@@ -373,7 +375,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       for (int m = 0; m < P1; ++m) *reinterpret_cast<float2*>(e + Rp::at(m, k2)) = y[m];
     }
     __syncthreads();  // rows transformed; the sensitivities of the step before were last read before it
-    if (t == 0) issue_s(c0);
+    if (t == 0 && ok) issue_s(c0);
 #pragma unroll 1
     for (int j = 0; j < CA; ++j) {
       const int cs = j * GA + g;
@@ -391,7 +393,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       if (GA == 1 && j == CA - 1) {
         tc::fence_proxy_async_smem();  // the in-place writes before the next step's copies
         __syncthreads();               // the slots are free
-        if (t == 0 && c0 + CS < op.nc) issue_g(c0 + CS);
+        if (t == 0 && ok && c0 + CS < op.nc) issue_g(c0 + CS);
       }
       if (on) DFT<P2, 1>::run(z);
       if (j == 0 && ok && !tc::mbar_wait(bar + 1, phase)) {
@@ -425,9 +427,13 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       }
       tc::fence_proxy_async_smem();
       __syncthreads();
-      if (t == 0 && c0 + CS < op.nc) issue_g(c0 + CS);
+      if (t == 0 && ok && c0 + CS < op.nc) issue_g(c0 + CS);
     }
   }
+  // after a time-out nothing more was requested: wait (bounded) for what was; of
+  // each barrier's two parities the completed one returns at once
+  if (t == 0 && !ok)
+    for (int i = 0; i < 4; ++i) tc::mbar_wait(bar + i / 2, i & 1, 200000000ull);
   float pq = 0.f;
   float* term = reinterpret_cast<float*>(ex);  // [RL P1][NIN] (GA > 1)
   if (ajob) {
