@@ -24,7 +24,7 @@ __global__ void k_dwt_rows_fwd(const float2* __restrict__ in, float2* __restrict
   float2 a = make_float2(0.f, 0.f), d = a;
   for (int m = 0; m < w.L; ++m) {
     int j = 2 * k + m;
-    if (j >= nxl) j -= nxl;
+    while (j >= nxl) j -= nxl;   // sides shorter than the filter wrap more than once
     const float2 v = row[j];
     a.x = fmaf(w.h[m], v.x, a.x);
     a.y = fmaf(w.h[m], v.y, a.y);
@@ -46,7 +46,7 @@ __global__ void k_dwt_cols_fwd(const float2* __restrict__ in, float2* __restrict
   float2 a = make_float2(0.f, 0.f), d = a;
   for (int m = 0; m < w.L; ++m) {
     int j = 2 * k + m;
-    if (j >= nyl) j -= nyl;
+    while (j >= nyl) j -= nyl;
     const float2 v = base[(size_t)j * n];
     a.x = fmaf(w.h[m], v.x, a.x);
     a.y = fmaf(w.h[m], v.y, a.y);
