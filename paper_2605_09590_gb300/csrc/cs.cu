@@ -555,7 +555,10 @@ void cs_shrink(FwdArgs f, float2* b0, float2* b1, int levels, int nb, const Wave
     const int m = n >> l0;
     const size_t sm = (size_t)2 * m * m * sizeof(float2);
     auto k = k_cs_core<TAN>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // always the limit of the largest core: it belongs to the function, and a context
+    // of another size in another thread must not lower it under this launch
+    constexpr int most = 2 * kCoreSide * kCoreSide * (int)sizeof(float2);
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     k<<<nb, kCoreThreads, sm, s>>>(buf[(l0 - 1) & 1], n, m, levels - l0, f.at, f.keep, f.tau, w);
   }
   for (int l = l0 - 1; l >= 1; --l)

@@ -1,0 +1,63 @@
+"""Contexts of different sizes in several host threads.
+
+The dynamic shared-memory limit of a kernel belongs to the function, not to the
+call or the thread: a launch that needs more than a limit which another thread
+has lowered is refused.  Every kernel whose request varies between contexts is
+used here by contexts of different sizes at once; each thread's results have the
+bits of the same calls alone.
+"""
+import threading
+
+import numpy as np
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def run_threads(targets):
+    errors = []
+
+    def guard(f):
+        try:
+            f()
+        except BaseException as e:  # noqa: BLE001 -- reported by the main thread
+            errors.append(e)
+
+    ts = [threading.Thread(target=guard, args=(f,)) for f in targets]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    if errors:
+        raise errors[0]
+
+
+def test_cs_reconstructions_of_different_sizes():
+    import paper_2605_09590_gb300 as pico
+    jobs = []
+    for n, levels, repeats in ((320, 4, 12), (64, 4, 40), (384, 4, 10), (64, 3, 40)):
+        S = synth.coil_maps(n, n, 2, 1)
+        mask = (np.random.default_rng(n).random((n, n)) < 0.6).astype(np.uint8)
+        op = pico.Operator(S, mask=mask, power_iters=10, max_batch=1)
+        x0 = torch.from_numpy(synth.phantom(n, 1).astype(np.complex64)).cuda().reshape(1, n, n)
+        b = op.forward(x0)[0].contiguous()
+        alone = torch.empty((n, n), dtype=torch.complex64, device="cuda")
+        pico.pico_cs_recon(op.ctx, b, 1e-3, 40, levels, alone)
+        op.sync()
+        jobs.append((op, b, levels, repeats, alone))
+    start = threading.Barrier(len(jobs))
+
+    def worker(op, b, levels, repeats, alone):
+        x = torch.empty_like(alone)
+        start.wait()
+        for _ in range(repeats):
+            pico.pico_cs_recon(op.ctx, b, 1e-3, 40, levels, x)
+        op.sync()
+        assert torch.equal(x, alone)
+
+    run_threads([lambda j=j: worker(*j) for j in jobs])
+    for j in jobs:
+        j[0].close()
