@@ -1233,16 +1233,22 @@ void launch_gram_apply_scale(const float* x, int ny, int nx, int nb, float* psca
   if (nb > 0) k_gram_apply_scale<<<nb, 256, 0, s>>>(x, (int64_t)2 * ny * nx, pscale);
 }
 
+constexpr size_t kGramStageBytes = 220 * 1024 - 2560;   // shared memory of all stages
+// alignment slack, barriers, TMEM slot, per-row beta and FP16 scale, per-column CG exchange slots (two FP64 sums per row)
+constexpr size_t gram_fixed_smem(int S) {
+  return 1024 + (3 * (size_t)S + 9) * 8 + 16 + 2 * kGramRows * 4 + 2 * kGramRows * 8 + 64;
+}
+constexpr size_t kGramSmemMax = gram_fixed_smem(8) + kGramStageBytes;
+
 size_t gram_smem(int ny, int kc, bool f16, int* stages) {
   const int nt = gram_tile(ny);
   const size_t stage = f16 ? 4 * (size_t)kGramRows * 16 * 4 + 4 * (size_t)kGramRows * 32 + 4 * (size_t)nt * 32
                            : 4 * (size_t)kGramRows * kc * 4 + 4 * (size_t)nt * kc * 4;
-  int S = (int)((220 * 1024 - 2560) / stage);
+  int S = (int)(kGramStageBytes / stage);
   if (S > 8) S = 8;
-  if (S < 2) S = 2;
+  if (S < 2) S = 2;   // two stages of the largest tile (256 rows, KC = 16) fit
   *stages = S;
-  // barriers, TMEM slot, per-row beta and FP16 scale, per-column CG exchange slots (two FP64 sums per row)
-  return 1024 + (size_t)S * stage + (3 * (size_t)S + 9) * 8 + 16 + 2 * kGramRows * 4 + 2 * kGramRows * 8 + 64;
+  return gram_fixed_smem(S) + (size_t)S * stage;
 }
 
 void launch_gram_normal(const GramOp& op, const CUtensorMap& mIn, const CUtensorMap& mPold, GramArgs g,
@@ -1257,15 +1263,17 @@ void launch_gram_normal(const GramOp& op, const CUtensorMap& mIn, const CUtensor
       f16 ? k_gram_normal<16, false, false, true>
           : op.kc == 16 ? (at ? k_gram_normal<16, true, false, false> : k_gram_normal<16, false, false, false>)
                         : (at ? k_gram_normal<8, true, false, false> : k_gram_normal<8, false, false, false>);
-  // the shared-memory opt-in is per device and kernel; cache it per (thread, device)
+  // the shared-memory opt-in is per device and kernel, not per call: always the
+  // most any size takes (a thread with a smaller image must not lower it under
+  // another's launches), set once per (thread, device)
   constexpr int kMaxDev = 16;
-  static thread_local size_t configured[kMaxDev][5] = {};
+  static thread_local bool configured[kMaxDev][5] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   const int ki = f16 ? 4 : (op.kc == 16 ? 0 : 2) + (at ? 1 : 0);
-  if (dev < 0 || dev >= kMaxDev || configured[dev][ki] < smem) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (dev >= 0 && dev < kMaxDev) configured[dev][ki] = smem;
+  if (dev < 0 || dev >= kMaxDev || !configured[dev][ki]) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmemMax);
+    if (dev >= 0 && dev < kMaxDev) configured[dev][ki] = true;
   }
   g.ny = op.ny;
   g.nx = op.nx;
@@ -1304,13 +1312,13 @@ bool launch_gram_colcg(const GramOp& op, const CUtensorMap& mIn, const CUtensorM
                                           : op.kc == 16 ? k_gram_normal<16, false, true, false>
                                                         : k_gram_normal<8, false, true, false>;
   constexpr int kMaxDev = 16;
-  static thread_local size_t configured[kMaxDev][3] = {};
+  static thread_local bool configured[kMaxDev][3] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   const int ki = f16 ? 2 : op.kc == 16 ? 0 : 1;
-  if (dev < 0 || dev >= kMaxDev || configured[dev][ki] < smem) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (dev >= 0 && dev < kMaxDev) configured[dev][ki] = smem;
+  if (dev < 0 || dev >= kMaxDev || !configured[dev][ki]) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmemMax);
+    if (dev >= 0 && dev < kMaxDev) configured[dev][ki] = true;
   }
   g.ny = op.ny;
   g.nx = op.nx;

@@ -61,3 +61,33 @@ def test_cs_reconstructions_of_different_sizes():
     run_threads([lambda j=j: worker(*j) for j in jobs])
     for j in jobs:
         j[0].close()
+
+
+def gram_op(ny, nx=32, nc=4):
+    import paper_2605_09590_gb300 as pico
+    op = pico.Operator(synth.coil_maps(ny, nx, nc, 1), mask=synth.mask_pe(ny, 2, 8), power_iters=0, max_batch=4)
+    op.set_tuning(gram_min_batch=1)
+    return op
+
+
+@pytest.mark.parametrize("solver", ["global", "columns"])
+def test_gram_kernels_after_a_smaller_context_of_another_thread(solver, monkeypatch):
+    """320 rows take 209 KB of shared memory per block, 256 rows 164 KB."""
+    monkeypatch.setenv("PICO_COLCG_PERSIST", "0")   # the per-update kernel
+    rng = np.random.default_rng(4)
+
+    def solve(op):
+        op.set_solver(solver)
+        x = rhs[op.ny]
+        y = op.cg(x, 6) if solver == "columns" else op.apply_normal(x)
+        op.sync()
+        return y
+
+    rhs = {ny: torch.from_numpy((rng.standard_normal((2, ny, 32)) + 1j * rng.standard_normal((2, ny, 32)))
+                                .astype(np.complex64)).cuda() for ny in (320, 256)}
+    large, small = gram_op(320), gram_op(256)
+    alone = solve(large)
+    run_threads([lambda: solve(small)])
+    assert torch.equal(solve(large), alone)
+    large.close()
+    small.close()
