@@ -1207,13 +1207,14 @@ void launch_gram_build(const float2* smaps, const uint8_t* mask_host, int nc, co
   }
   cudaMemcpyAsync(pbuf, P.data(), ny * sizeof(double2), cudaMemcpyHostToDevice, s);
   const size_t sbytes = (size_t)nc * ny * sizeof(float2);
+  constexpr int most = 200 * 1024;   // the limit set is the same for every size (see launch_gram_normal)
   if (op.f16) {
     // the FP16 form needs the column's sensitivities in shared memory (its scale bound)
-    cudaFuncSetAttribute(k_gram_build_smem<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sbytes);
+    cudaFuncSetAttribute(k_gram_build_smem<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     k_gram_build_smem<true><<<dim3(nx, (ny + 31) / 32), 256, sbytes, s>>>(smaps, pbuf, nc, ny, nx, op.nt, 16,
                                                                            op.G, op.gscale);
-  } else if (sbytes <= 200 * 1024) {
-    cudaFuncSetAttribute(k_gram_build_smem<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sbytes);
+  } else if (sbytes <= most) {
+    cudaFuncSetAttribute(k_gram_build_smem<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     k_gram_build_smem<false><<<dim3(nx, (ny + 31) / 32), 256, sbytes, s>>>(smaps, pbuf, nc, ny, nx, op.nt,
                                                                             op.kc, op.G, op.gscale);
   } else {

@@ -91,3 +91,32 @@ def test_gram_kernels_after_a_smaller_context_of_another_thread(solver, monkeypa
     assert torch.equal(solve(large), alone)
     large.close()
     small.close()
+
+
+def test_gram_setups_of_different_sizes():
+    """The set-up keeps a column's sensitivities in shared memory: coils x rows x 8 bytes.
+
+    Changing the contraction depth builds the operator anew."""
+    shapes = ((128, 3), (256, 64), (128, 5), (320, 70))
+    start = threading.Barrier(len(shapes))
+    rng = np.random.default_rng(5)
+    cases = []
+    for ny, nc in shapes:
+        x = torch.from_numpy((rng.standard_normal((1, ny, 16)) + 1j * rng.standard_normal((1, ny, 16)))
+                             .astype(np.complex64)).cuda()
+        op = gram_op(ny, 16, nc)
+        cases.append((op, x, op.apply_normal(x)))
+        op.sync()
+
+    def worker(op, x, alone):
+        start.wait()
+        for _ in range(1000):
+            op.set_tuning(gram_kc=8)
+            op.set_tuning(gram_kc=16)
+        y = op.apply_normal(x)
+        op.sync()
+        assert torch.equal(y, alone)
+
+    run_threads([lambda c=c: worker(*c) for c in cases])
+    for c in cases:
+        c[0].close()
