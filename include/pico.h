@@ -436,8 +436,10 @@ pico_status pico_tune_select(const double* times_us, int32_t max_batch, int32_t 
 /* Wait for all work of the context and report its asynchronous status:
  * PICO_E_CUDA for a CUDA error; otherwise every pending class is named in
  * pico_last_error and the status is PICO_E_TIMEOUT if a kernel's bounded
- * pipeline wait (the tensor-core Gram operator, the TMA-staged Toeplitz column
- * pass) gave up, else PICO_E_BREAKDOWN if a CG system broke down (a non-finite
+ * wait gave up (copies and accumulators of the tensor-core Gram operator and
+ * of the whole-solve per-column CG, staged copies of the three Toeplitz /
+ * 2-D-mask passes and of the Cartesian row adjoint, the exchange of the on-chip
+ * whole-image CG; the text gives its code and name), else PICO_E_BREAKDOWN if a CG system broke down (a non-finite
  * residual -- NaN or Inf in a right-hand side or the operator -- or
  * p^H (M + lam) p <= 0) since the last pico_sync.  Broken-down systems keep the
  * iterate reached before the breakdown (x = 0 for a non-finite right-hand

@@ -1699,7 +1699,7 @@ pico_status pico_sync(pico_ctx* c) {
   if (broken) cudaMemsetAsync(c->status, 0, s.size() * sizeof(int), c->stream);
   if ((e || broken) && cudaStreamSynchronize(c->stream) != cudaSuccess) return cuda_check(c, "pico_sync");
   std::string msg;
-  if (e) msg = "a kernel's bounded pipeline wait timed out (code " + std::to_string(e) + ")";
+  if (e) msg = "a kernel's bounded pipeline wait timed out (code " + std::to_string(e) + ": " + pico::wait_name(e) + ")";
   if (broken) {
     if (!msg.empty()) msg += "; ";
     msg += "CG breakdown (non-finite residual or p^H (M + lam) p <= 0) in " + std::to_string(broken) +

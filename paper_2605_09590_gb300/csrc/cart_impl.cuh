@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
   for (int c0 = 0; c0 < op.nc; c0 += CS, phase ^= 1) {
     if (ok && !tc::mbar_wait(bar, phase)) {  // reported by pico_sync; the block runs on so that its barriers pair up
       ok = false;
-      if (err) atomicCAS(err, 0, 13);
+      if (err) atomicCAS(err, 0, kWaitRowAdjoint);
     }
     if (c0 + cb < op.nc) {
       float2 y[M1];
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       if (on) DFT<M2, 1>::run(z);
       if (j == 0 && ok && !tc::mbar_wait(bar + 1, phase)) {
         ok = false;
-        if (err) atomicCAS(err, 0, 13);
+        if (err) atomicCAS(err, 0, kWaitRowAdjoint);
       }
       if (on) {
         const float2* S = sst + (j * RL + ra) * M + n1;

@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2)
 #pragma unroll
         for (int m = 0; m < 4; ++m) ready = ready && (unsigned)(w0[m] >> 32) == seq && (unsigned)(w1[m] >> 32) == seq;
         if (!ready && global_ns() - t0 > 2000000000ull) {
-          if (err) atomicCAS(err, 0, 11);
+          if (err) atomicCAS(err, 0, kWaitExchange);
           ok = false;
           break;
         }

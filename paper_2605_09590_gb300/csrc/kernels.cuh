@@ -12,6 +12,33 @@ constexpr int kVecThreads = 256;
 constexpr int kVecPerThread = 4;
 constexpr int kVecPerBlock = kVecThreads * kVecPerThread;
 
+// What a kernel writes to the context's error word when a bounded wait gives up
+// (the first one stays; pico_sync names it): one code per wait, or per kernel
+// whose waits say the same.
+enum WaitCode : int {
+  kWaitGramFirst = 1,  // gram.cu, 1-7: stages, accumulator and tile copies
+  kWaitGramLast = 7,
+  kWaitToepCols = 10,
+  kWaitExchange = 11,
+  kWaitToepRowsInv = 12,
+  kWaitRowAdjoint = 13,
+  kWaitToepRowsFwd = 14,
+  kWaitPersistFirst = 21,  // colcg_persist.cu, 21-25
+  kWaitPersistLast = 25,
+};
+inline const char* wait_name(int code) {
+  if (code >= kWaitGramFirst && code <= kWaitGramLast) return "Gram operator";
+  if (code >= kWaitPersistFirst && code <= kWaitPersistLast) return "whole-solve per-column CG";
+  switch (code) {
+    case kWaitToepCols: return "Toeplitz / 2-D-mask column pass";
+    case kWaitExchange: return "whole-image CG exchange on chip";
+    case kWaitToepRowsInv: return "Toeplitz / 2-D-mask inverse row pass";
+    case kWaitRowAdjoint: return "Cartesian row adjoint";
+    case kWaitToepRowsFwd: return "Toeplitz / 2-D-mask forward row pass";
+    default: return "unknown wait";
+  }
+}
+
 // Batched CG state (Eq. 6 solved for many right-hand sides at once).
 // Scalars are kept per iteration so that every value is written once:
 // rr(b, it) = sum_j rr_part[(b*(itmax+1) + it)*PB + j]   (r^H r before update it)

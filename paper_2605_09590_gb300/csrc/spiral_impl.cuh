@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
   for (int c0 = 0; c0 < op.nc; c0 += CS, phase ^= 1) {
     if (ok && !tc::mbar_wait(bar, phase)) {  // reported by pico_sync; the block runs on so that its barriers pair up
       ok = false;
-      if (op.err) atomicCAS(op.err, 0, 11);
+      if (op.err) atomicCAS(op.err, 0, kWaitToepRowsFwd);
     }
     if (ajob) {
 #pragma unroll
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(ColsW<P1, P2>::NT, (ColsW<P1, P2>::blocks(PAD 
     if (t == 0) {
       bool ok = tc::mbar_wait(bar, phase);
       if (!ok) {
-        if (op.err) atomicCAS(op.err, 0, 10);
+        if (op.err) atomicCAS(op.err, 0, kWaitToepCols);
         tc::mbar_wait(bar, phase);
       }
       *arrived = ok ? 1 : 0;
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
   for (int c0 = 0; c0 < op.nc; c0 += CS, phase ^= 1) {
     if (ok && !tc::mbar_wait(bar, phase)) {  // reported by pico_sync; the block runs on so that its barriers pair up
       ok = false;
-      if (op.err) atomicCAS(op.err, 0, 12);
+      if (op.err) atomicCAS(op.err, 0, kWaitToepRowsInv);
     }
     if (c0 + cb < op.nc) {
       float2 y[P1];
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
       if (on) DFT<P2, 1>::run(z);
       if (j == 0 && ok && !tc::mbar_wait(bar + 1, phase)) {
         ok = false;
-        if (op.err) atomicCAS(op.err, 0, 12);
+        if (op.err) atomicCAS(op.err, 0, kWaitToepRowsInv);
       }
       if (GA == 1) {
         if (on) {
