@@ -592,7 +592,7 @@ void launch_row_adjoint_t(const CartOp& op, const float2* G, float2* out, int nb
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     CUtensorMap mG{};
     if (op.ny % kRowLines == 0 && (int64_t)nb * (op.ny / kRowLines) > 2 * nsm &&
-        encode_row_map(&mG, G, M1, M2, (int64_t)nb * op.nc * op.ny, 1)) {
+        encode_row_map(&mG, G, M1, M2, (int64_t)nb * op.nc * op.ny)) {
       const size_t sm = Rp::smem(op.nx);
       auto k = k_row_adjoint_v<M1, M2, NT>;
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);

@@ -52,19 +52,6 @@ __device__ __forceinline__ void colb_store(const float2 (&y)[P1], int k2, int ln
 #pragma unroll
   for (int m = 0; m < P1; ++m) buf[(k2 * P1 + m) * LS + ln] = y[m];
 }
-// inverse DFT_P1 of a b-job and the conjugate twiddle, stored for the a-jobs
-template <int P1, int P2, int LS = kLines>
-__device__ __forceinline__ void colb_inv_store(float2 (&y)[P1], int k2, int ln, float2* buf, const float2* tws) {
-  DFT<P1, 1>::run(y);
-#pragma unroll
-  for (int m = 0; m < P1; ++m) buf[(k2 * P1 + m) * LS + ln] = m == 0 ? y[0] : cmul_cb(y[m], tws[m * k2]);
-}
-template <int P1, int P2, int SIGN, int LS = kLines>
-__device__ __forceinline__ void cola_load(float2 (&z)[P2], int n1, int ln, const float2* buf) {
-#pragma unroll
-  for (int k = 0; k < P2; ++k) z[k] = buf[(k * P1 + n1) * LS + ln];
-  DFT<P2, SIGN>::run(z);
-}
 
 // DFT_P of which only the first NZ inputs can be non-zero (zero-padded lines)
 template <int P, int SIGN, int NZ>
@@ -93,20 +80,6 @@ __device__ __forceinline__ void rowb_load(float2 (&y)[P1], int k2, int ln, const
 #pragma unroll
   for (int m = 0; m < P1; ++m) y[m] = buf[(ln * P2 + k2) * LD + m];
   DFT<P1, SIGN>::run(y);
-}
-template <int P1, int P2>
-__device__ __forceinline__ void rowb_inv_store(float2 (&y)[P1], int k2, int ln, float2* buf, const float2* tws) {
-  constexpr int LD = Split<P1, P2>::LD;
-  DFT<P1, 1>::run(y);
-#pragma unroll
-  for (int m = 0; m < P1; ++m) buf[(ln * P2 + k2) * LD + m] = m == 0 ? y[0] : cmul_cb(y[m], tws[m * k2]);
-}
-template <int P1, int P2>
-__device__ __forceinline__ void rowa_inv_load(float2 (&z)[P2], int n1, int ln, const float2* buf) {
-  constexpr int LD = Split<P1, P2>::LD;
-#pragma unroll
-  for (int k = 0; k < P2; ++k) z[k] = buf[(ln * P2 + k) * LD + n1];
-  DFT<P2, 1>::run(z);
 }
 
 }  // namespace pico

@@ -1166,12 +1166,12 @@ bool encode_plane_map(CUtensorMap* m, const void* base, int rows, int L, int64_t
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool encode_row_map(CUtensorMap* m, const void* base, int P1, int P2, int64_t rows, int box_rows) {
+bool encode_row_map(CUtensorMap* m, const void* base, int P1, int P2, int64_t rows) {
   EncodeTiledFn enc = encode_fn();
   if (!enc || !base || (reinterpret_cast<uintptr_t>(base) & 15) || (P2 != 8 && P2 != 16) || P1 > 256) return false;
   cuuint64_t dims[3] = {(cuuint64_t)P2, (cuuint64_t)P1, (cuuint64_t)rows};
   cuuint64_t strides[2] = {(cuuint64_t)P2 * 8, (cuuint64_t)P1 * P2 * 8};
-  cuuint32_t box[3] = {(cuuint32_t)P2, (cuuint32_t)P1, (cuuint32_t)box_rows}, es[3] = {1, 1, 1};
+  cuuint32_t box[3] = {(cuuint32_t)P2, (cuuint32_t)P1, 1}, es[3] = {1, 1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_INT64, 3, const_cast<void*>(base), dims, strides, box, es,
              CU_TENSOR_MAP_INTERLEAVE_NONE, P2 == 16 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;

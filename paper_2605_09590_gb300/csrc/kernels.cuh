@@ -271,9 +271,9 @@ constexpr int kRowLines = 4;
 // 3-D tensor map over `planes` planes of rows x L complex64 values (8-byte
 // elements), boxes of `cols` x `box_rows` values (the column pass's staging)
 bool encode_plane_map(CUtensorMap* m, const void* base, int rows, int L, int64_t planes, int cols, int box_rows);
-// 3-D tensor map over grid rows of P1 x P2 complex64 values, boxes of box_rows
-// rows swizzled by their P2 values (the inverse row pass's exchange layout)
-bool encode_row_map(CUtensorMap* m, const void* base, int P1, int P2, int64_t rows, int box_rows);
+// 3-D tensor map over grid rows of P1 x P2 complex64 values, boxes of one row
+// swizzled by its P2 values (the inverse row pass's exchange layout)
+bool encode_row_map(CUtensorMap* m, const void* base, int P1, int P2, int64_t rows);
 bool spiral_supported(int n, int* P1, int* P2);
 bool grid_split(int L, int* P1, int* P2);  // split of a 2-D pass length (Toeplitz or 2-D Cartesian)
 void launch_toep_h(const float* traj, int64_t M, int n, float2* c, cudaStream_t s);

@@ -10,7 +10,7 @@ template <int P1, int P2>
 bool launch_toep_normal_t(const SpiralOp&, const float2*, float2*, float2*, int, float, const CgArgs*, int,
                           cudaStream_t);
 template <int P1, int P2>
-void launch_fft2_t(float2*, const float2*, int, int, bool, cudaStream_t);
+void launch_fft2_t(float2*, const float2*, bool, cudaStream_t);
 template <int P1, int P2>
 void launch_grid_rows_adjoint_t(const SpiralOp&, float2*, int, cudaStream_t);
 template <int P1, int P2>
@@ -278,8 +278,8 @@ void launch_toep_h(const float* traj, int64_t M, int n, float2* c, cudaStream_t 
 void launch_toep_fft2(const SpiralOp& op, float2* c, cudaStream_t s) {
 #define PICO_CASE(LL, A, B)                               \
   if (op.P1 == A && op.P2 == B) {                         \
-    launch_fft2_t<A, B>(c, op.tw2, 1, -1, true, s);       \
-    launch_fft2_t<A, B>(c, op.tw2, 1, -1, false, s);      \
+    launch_fft2_t<A, B>(c, op.tw2, true, s);              \
+    launch_fft2_t<A, B>(c, op.tw2, false, s);             \
     return;                                               \
   }
   PICO_GRID_SIZES(PICO_CASE)

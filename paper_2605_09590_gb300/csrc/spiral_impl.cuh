@@ -464,10 +464,10 @@ __global__ void __launch_bounds__(NT, 512 / NT)
 }
 
 // ---------------------------------------------------------------------------
-// Generic in-place FFTs of all rows / all columns of [planes][L][L] grids
+// In-place forward FFTs of all rows / all columns of an L x L grid (set-up)
 // ---------------------------------------------------------------------------
-template <int P1, int P2, int SIGN>
-__global__ void __launch_bounds__(Split<P1, P2>::NT, 1) k_fft_rows(float2* __restrict__ data, const float2* tw2) {
+template <int P1, int P2>
+__global__ void __launch_bounds__(Split<P1, P2>::NT, 1) k_fft_rows(float2* __restrict__ plane, const float2* tw2) {
   constexpr int L = P1 * P2;
   constexpr int NT = Split<P1, P2>::NT;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -476,7 +476,6 @@ __global__ void __launch_bounds__(Split<P1, P2>::NT, 1) k_fft_rows(float2* __res
   const int t = threadIdx.x;
   for (int i = t; i < L; i += NT) tws[i] = tw2[i];
   __syncthreads();
-  float2* __restrict__ plane = data + (size_t)blockIdx.y * L * L;
   const int ra = t / P1, n1 = t % P1;
   const int rb = t / P2, k2 = t % P2;
   if (t < kLines * P1) {
@@ -484,20 +483,20 @@ __global__ void __launch_bounds__(Split<P1, P2>::NT, 1) k_fft_rows(float2* __res
     const float2* row = plane + (size_t)(blockIdx.x * kLines + ra) * L;
 #pragma unroll
     for (int n2 = 0; n2 < P2; ++n2) z[n2] = row[n1 + P1 * n2];
-    rowa_store<P1, P2, SIGN>(z, n1, ra, buf, tws);
+    rowa_store<P1, P2, -1>(z, n1, ra, buf, tws);
   }
   __syncthreads();
   if (t < kLines * P2) {
     float2 y[P1];
-    rowb_load<P1, P2, SIGN>(y, k2, rb, buf);
+    rowb_load<P1, P2, -1>(y, k2, rb, buf);
     float2* row = plane + (size_t)(blockIdx.x * kLines + rb) * L;
 #pragma unroll
     for (int k1 = 0; k1 < P1; ++k1) row[k2 + P2 * k1] = y[k1];
   }
 }
 
-template <int P1, int P2, int SIGN>
-__global__ void __launch_bounds__(Split<P1, P2>::NT, 1) k_fft_cols(float2* __restrict__ data, const float2* tw2) {
+template <int P1, int P2>
+__global__ void __launch_bounds__(Split<P1, P2>::NT, 1) k_fft_cols(float2* __restrict__ plane, const float2* tw2) {
   constexpr int L = P1 * P2;
   constexpr int NT = Split<P1, P2>::NT;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -506,20 +505,19 @@ __global__ void __launch_bounds__(Split<P1, P2>::NT, 1) k_fft_cols(float2* __res
   const int t = threadIdx.x;
   for (int i = t; i < L; i += NT) tws[i] = tw2[i];
   __syncthreads();
-  float2* __restrict__ plane = data + (size_t)blockIdx.y * L * L;
   const int ln = t % kLines, job = t / kLines;
   const int kx = blockIdx.x * kLines + ln;
   if (job < P1) {
     float2 z[P2];
 #pragma unroll
     for (int n2 = 0; n2 < P2; ++n2) z[n2] = plane[(size_t)(job + P1 * n2) * L + kx];
-    cola_store<P1, P2, SIGN>(z, job, ln, buf, tws);
+    cola_store<P1, P2, -1>(z, job, ln, buf, tws);
   }
   __syncthreads();
   if (job < P2) {
     float2 y[P1];
     colb_load<P1, P2>(y, job, ln, buf);
-    DFT<P1, SIGN>::run(y);
+    DFT<P1, -1>::run(y);
 #pragma unroll
     for (int k1 = 0; k1 < P1; ++k1) plane[(size_t)(job + P2 * k1) * L + kx] = y[k1];
   }
@@ -657,7 +655,7 @@ bool toep_rows_inv_launch(const SpiralOp& op, const float2* x, float2* y, const 
                           const CgArgs* a, int it, cudaStream_t s) {
   using Rp = RowPass<P1, P2, NT>;
   CUtensorMap mG{};
-  if (!encode_row_map(&mG, G, P1, P2, (int64_t)nb * op.nc * op.n, 1)) return false;
+  if (!encode_row_map(&mG, G, P1, P2, (int64_t)nb * op.nc * op.n)) return false;
   const size_t sm = Rp::smem(op.n);
   const dim3 grow(op.n / Rp::RL, nb);
   auto k3 = a ? k_toep_rows_inv<P1, P2, true, PAD, NT> : k_toep_rows_inv<P1, P2, false, PAD, NT>;
@@ -719,19 +717,19 @@ bool launch_toep_normal_t(const SpiralOp& op, const float2* x, float2* y, float2
 }
 
 template <int P1, int P2>
-void launch_fft2_t(float2* data, const float2* tw2, int planes, int sign, bool rows, cudaStream_t s) {
+void launch_fft2_t(float2* plane, const float2* tw2, bool rows, cudaStream_t s) {
   using Sp = Split<P1, P2>;
   constexpr int L = P1 * P2;
   if (rows) {
     const size_t sm = Sp::row_buf + L * sizeof(float2);
-    auto k = sign < 0 ? k_fft_rows<P1, P2, -1> : k_fft_rows<P1, P2, 1>;
+    auto k = k_fft_rows<P1, P2>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k<<<dim3(L / kLines, planes), Sp::NT, sm, s>>>(data, tw2);
+    k<<<L / kLines, Sp::NT, sm, s>>>(plane, tw2);
   } else {
     const size_t sm = Sp::col_buf + L * sizeof(float2);
-    auto k = sign < 0 ? k_fft_cols<P1, P2, -1> : k_fft_cols<P1, P2, 1>;
+    auto k = k_fft_cols<P1, P2>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k<<<dim3(L / kLines, planes), Sp::NT, sm, s>>>(data, tw2);
+    k<<<L / kLines, Sp::NT, sm, s>>>(plane, tw2);
   }
 }
 
