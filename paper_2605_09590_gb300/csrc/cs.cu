@@ -218,7 +218,12 @@ __global__ void k_axpy_bcast(float2* __restrict__ x, const float2* __restrict__ 
 // kernels (L2 / HBM) for many images and by the launches for one.
 // ---------------------------------------------------------------------------
 constexpr int kTapMax = 8;
-constexpr int kFuseTX = 32;        // coefficients per tile and band along x
+// Coefficients per tile and band.  8 rows (halo 1.5x, 24 KB of shared memory per
+// block) rather than 16 (1.3x, 41 KB): more and smaller blocks per SM outweigh the
+// halo for every size and batch tried (wavelet kernels of one iteration, 320 x 320:
+// 96 images 254 against 286 us, 4 images 41 against 50 us; 64 x 64, 512 images 68
+// against 73 us).
+constexpr int kFuseTX = 32, kFuseTY = 8;
 constexpr int kFuseThreads = 256;
 constexpr int kLoadAhead = 6;      // global loads in flight per thread and operand
 
@@ -263,10 +268,10 @@ __device__ __forceinline__ float2 cs_threshold(float2 v, size_t i, const float2*
   return soft1(v, tau);
 }
 
-// One analysis level on tiles of TY x kFuseTX coefficients per band.
-template <int LOAD, bool TAN, int TY>
+// One analysis level on tiles of kFuseTY x kFuseTX coefficients per band.
+template <int LOAD, bool TAN>
 __global__ void __launch_bounds__(kFuseThreads) k_cs_fwd(FwdArgs f, Wavelet w) {
-  constexpr int TX = kFuseTX, IY = 2 * TY + kTapMax - 2, IX = 2 * TX + kTapMax - 2;
+  constexpr int TX = kFuseTX, TY = kFuseTY, IY = 2 * TY + kTapMax - 2, IX = 2 * TX + kTapMax - 2;
   __shared__ __align__(16) float2 in[IY][IX];
   __shared__ float2 mid[IY][2 * TX];   // row analysis: [approximation | detail]
   const int t = threadIdx.x, b = blockIdx.z, n = f.n, m = f.m, half = m / 2;
@@ -358,10 +363,10 @@ __device__ __forceinline__ void cs_store(const InvArgs& f, size_t o, float2 v) {
   f.o0[o] = v;
 }
 
-// One synthesis level on tiles of 2 TY x 2 kFuseTX outputs.
-template <int STORE, int TY>
+// One synthesis level on tiles of 2 kFuseTY x 2 kFuseTX outputs.
+template <int STORE>
 __global__ void __launch_bounds__(kFuseThreads) k_cs_inv(InvArgs f, Wavelet w) {
-  constexpr int TX = kFuseTX, HB = kTapMax / 2 - 1, CY = TY + HB, CX = TX + HB;
+  constexpr int TX = kFuseTX, TY = kFuseTY, HB = kTapMax / 2 - 1, CY = TY + HB, CX = TX + HB;
   __shared__ float2 in[2][CY][2 * CX];     // [rows: approximation | detail][k][columns: approximation | detail]
   __shared__ float2 mid[2 * TY][2 * CX];   // column synthesis
   const int t = threadIdx.x, b = blockIdx.z, n = f.n, m = f.m, half = m / 2;
@@ -512,22 +517,8 @@ __global__ void __launch_bounds__(kCoreThreads) k_cs_core(float2* data, int n, i
   for (int e = t; e < m * m; e += kCoreThreads) img[(size_t)(e / m) * n + e % m] = A[e];
 }
 
-template <int LOAD, bool TAN>
-void fwd_level(const FwdArgs& f, int nb, const Wavelet& w, cudaStream_t s) {
-  const int half = f.m / 2, bx = (half + kFuseTX - 1) / kFuseTX;
-  // tiles of 16 coefficient rows (halo 1.3x) once they fill the device, else of 8 (1.5x, twice the blocks)
-  if ((int64_t)bx * ((half + 15) / 16) * nb >= 1024)
-    k_cs_fwd<LOAD, TAN, 16><<<dim3(bx, (half + 15) / 16, nb), kFuseThreads, 0, s>>>(f, w);
-  else
-    k_cs_fwd<LOAD, TAN, 8><<<dim3(bx, (half + 7) / 8, nb), kFuseThreads, 0, s>>>(f, w);
-}
-template <int STORE>
-void inv_level(const InvArgs& f, int nb, const Wavelet& w, cudaStream_t s) {
-  const int half = f.m / 2, bx = (half + kFuseTX - 1) / kFuseTX;
-  if ((int64_t)bx * ((half + 15) / 16) * nb >= 1024)
-    k_cs_inv<STORE, 16><<<dim3(bx, (half + 15) / 16, nb), kFuseThreads, 0, s>>>(f, w);
-  else
-    k_cs_inv<STORE, 8><<<dim3(bx, (half + 7) / 8, nb), kFuseThreads, 0, s>>>(f, w);
+inline dim3 level_tiles(int m, int nb) {
+  return dim3((m / 2 + kFuseTX - 1) / kFuseTX, (m / 2 + kFuseTY - 1) / kFuseTY, nb);
 }
 
 // Coefficients of y (from cs_load<LOAD>) thresholded and transformed back:
@@ -543,13 +534,13 @@ void cs_shrink(FwdArgs f, float2* b0, float2* b1, int levels, int nb, const Wave
   f.m = n;
   f.dst = b0;
   f.last = levels == 1;
-  fwd_level<LOAD, TAN>(f, nb, w, s);
+  k_cs_fwd<LOAD, TAN><<<level_tiles(f.m, nb), kFuseThreads, 0, s>>>(f, w);
   for (int l = 1; l < l0; ++l) {
     f.a = buf[(l - 1) & 1];
     f.dst = buf[l & 1];
     f.m = n >> l;
     f.last = l == levels - 1;
-    fwd_level<kLoadPlain, TAN>(f, nb, w, s);
+    k_cs_fwd<kLoadPlain, TAN><<<level_tiles(f.m, nb), kFuseThreads, 0, s>>>(f, w);
   }
   if (l0 < levels) {
     const int m = n >> l0;
@@ -562,7 +553,8 @@ void cs_shrink(FwdArgs f, float2* b0, float2* b1, int levels, int nb, const Wave
     k<<<nb, kCoreThreads, sm, s>>>(buf[(l0 - 1) & 1], n, m, levels - l0, f.at, f.keep, f.tau, w);
   }
   for (int l = l0 - 1; l >= 1; --l)
-    inv_level<kStorePlain>(InvArgs{n, n >> l, buf[l & 1], buf[(l - 1) & 1], nullptr, 0.f}, nb, w, s);
+    k_cs_inv<kStorePlain><<<level_tiles(n >> l, nb), kFuseThreads, 0, s>>>(
+        InvArgs{n, n >> l, buf[l & 1], buf[(l - 1) & 1], nullptr, 0.f}, w);
 }
 
 __global__ void k_scale(float2* __restrict__ x, float s, int64_t n) {
@@ -672,7 +664,7 @@ void launch_cs_iter(const float2* z, const float2* Mz, const float2* rhs, int64_
     cs_shrink<kLoadGrad, true>(f, b0, b1, levels, nb, w, s);
   else
     cs_shrink<kLoadGrad, false>(f, b0, b1, levels, nb, w, s);
-  inv_level<kStoreMomentum>(InvArgs{n, n, b0, x, zout, c}, nb, w, s);
+  k_cs_inv<kStoreMomentum><<<level_tiles(n, nb), kFuseThreads, 0, s>>>(InvArgs{n, n, b0, x, zout, c}, w);
 }
 
 void launch_vjp_iter(const float2* yb, const float2* Myb, float inv_lc, const float2* xb, float c_prev, float c,
@@ -680,7 +672,7 @@ void launch_vjp_iter(const float2* yb, const float2* Myb, float inv_lc, const fl
                      int n, int levels, int nb, const Wavelet& w, cudaStream_t s) {
   FwdArgs f{n, n, yb, Myb, xb, 0, inv_lc, 1.f + c, c_prev, znew, b0, at, nullptr, tau, 0};
   cs_shrink<kLoadVjp, true>(f, b0, b1, levels, nb, w, s);
-  inv_level<kStoreVjp>(InvArgs{n, n, b0, yout, ysum, 0.f}, nb, w, s);
+  k_cs_inv<kStoreVjp><<<level_tiles(n, nb), kFuseThreads, 0, s>>>(InvArgs{n, n, b0, yout, ysum, 0.f}, w);
 }
 void launch_scale(float2* x, float sc, int64_t n, int nb, cudaStream_t s) {
   k_scale<<<dim3(blocks(n), nb), 256, 0, s>>>(x, sc, n);
