@@ -684,8 +684,13 @@ bool toep_cols_launch(const SpiralOp& op, float2* G, int nb, const int* done, in
 // Threads per block of the row passes: 128 (64 where the a-jobs of four rows fit
 // in 64), four (eight) blocks per SM, once the row blocks fill the device; below
 // that more coils at once per block, which shortens the serial walk over the
-// coils -- 256 threads while all blocks are resident at two per SM, 512 while
-// one per SM is enough.
+// coils -- 256 threads while every block is resident (two per SM; one where the
+// shared memory of 480 x 480 masks allows no more), 512 while one per SM is enough.
+// Both row passes with 512 / 256 / 128 threads, 152 SMs: 240 x 240 spiral, 20 coils,
+// 120 row blocks 31 / 34 / 42 us, 180 blocks 59 / 53 / 57, 300 blocks 67 / 57 / 63,
+// 360 blocks 99 / 96 / 78; 320 x 320 mask, 15 coils, 80 blocks 21 / 25 / 31, 240 blocks
+// 41 / 36 / 40, 320 blocks 59 / 55 / 49; 480 x 480 mask, 8 coils, 120 blocks 256 / 128
+// threads 20 / 23 us, 240 blocks 36 / 31.
 template <int P1, int P2, bool PAD, int NT>
 bool toep_normal_nt(const SpiralOp& op, const float2* x, float2* y, float2* G, int nb, float lam, const CgArgs* a,
                     int it, int nsm, cudaStream_t s) {
@@ -705,7 +710,8 @@ bool toep_normal_impl(const SpiralOp& op, const float2* x, float2* y, float2* G,
   constexpr bool wide = RowPass<P1, P2, 512>::smem(PAD ? P1 * P2 / 2 : P1 * P2) <= 227 * 1024;
   if constexpr (wide)
     if (blocks <= nsm) return toep_normal_nt<P1, P2, PAD, 512>(op, x, y, G, nb, lam, a, it, nsm, s);
-  if (blocks <= 2 * nsm) return toep_normal_nt<P1, P2, PAD, 256>(op, x, y, G, nb, lam, a, it, nsm, s);
+  constexpr int resident = 2 * (RowPass<P1, P2, 256>::smem(PAD ? P1 * P2 / 2 : P1 * P2) + 1024) <= 228 * 1024 ? 2 : 1;
+  if (blocks <= resident * nsm) return toep_normal_nt<P1, P2, PAD, 256>(op, x, y, G, nb, lam, a, it, nsm, s);
   return toep_normal_nt<P1, P2, PAD, (kRowLines * P1 <= 64 ? 64 : 128)>(op, x, y, G, nb, lam, a, it, nsm, s);
 }
 
