@@ -445,7 +445,10 @@ __global__ void __launch_bounds__(RowShape<M1, M2>::NT, (RowShape<M1, M2>::NT <=
 // in the swizzled exchange layout, sensitivity rows by bulk copies, both while
 // other work runs, and four blocks share an SM.  256 replicas of 15 coils at
 // 320 x 320: k_row_adjoint (16 rows, two 320-thread blocks per SM, strided
-// twiddle look-ups) 1042 us, this 922 us; the hybrid's 3.15 GB take 464 us.
+// twiddle look-ups) 1042 us, this 922 us; the hybrid's 3.15 GB take 464 us.  It
+// spills (40 bytes a thread at 320, 88 at 384); three blocks per SM, which do not,
+// take 998 us against 931 us there and 366 against 352 us for 128 replicas of
+// 8 coils at 384 x 384.
 template <int M1, int M2, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT)
     k_row_adjoint_v(CartOp op, const __grid_constant__ CUtensorMap mG, float2* __restrict__ out, int* err) {
@@ -583,8 +586,11 @@ void launch_col_pmr_t(const CartOp& op, float2* G, int nb, uint64_t seed, int64_
 template <int M1, int M2>
 void launch_row_adjoint_t(const CartOp& op, const float2* G, float2* out, int nb, int* err, cudaStream_t s) {
   if constexpr (M2 >= 8) {
-    // four-row blocks once they fill the device (two per SM); few of them are
-    // quicker as blocks of 16 rows and 16 M1 threads
+    // four-row blocks once they fill the device (two per SM).  Below that the two lie
+    // close for one to three coils, where 16-row blocks are up to 15 % quicker (eight
+    // images of 320 x 320, one coil: 6.3 against 7.3 us); with more coils four-row blocks
+    // are the quicker ones there too (one image of 15 coils: 17 against 38 us, eight
+    // images of 192 x 192, 8 coils: 12.8 against 13.0), so a line by coils would lie better
     constexpr int NT = kRowLines * M1 <= 64 ? 64 : 128;
     using Rp = RowPass<M1, M2, NT>;
     int dev = 0, nsm = 0;

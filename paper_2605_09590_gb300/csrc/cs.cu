@@ -210,12 +210,13 @@ __global__ void k_axpy_bcast(float2* __restrict__ x, const float2* __restrict__ 
 // instead of one launch per direction and level and one per element-wise step:
 // 5 launches per iteration of a 4-level transform at 320 x 320 in place of
 // 19-20, the images cross memory once per level and direction instead of twice,
-// and the element-wise steps take no pass of their own (320 x 320, 48 images:
-// 367 us of such passes per iteration before, 205 us as fused; one image: 84 us
-// before).  The arithmetic of every value is that of the
+// and the element-wise steps take no pass of their own (320 x 320, kernel time of
+// an iteration: 48 images 367 us as single passes, 147 us fused; one image 84 and
+// 37 us).  The arithmetic of every value is that of the
 // single passes (rows before columns in the analysis, columns before rows in the
-// synthesis, taps in the same order).  Bound by the loads of the level-0
-// kernels (L2 / HBM) for many images and by the launches for one.
+// synthesis, taps in the same order).  Bound by shared memory, local memory (the
+// synthesis taps below) and the loads of the level-0 kernels for many images, by
+// the latency of each launch for one.
 // ---------------------------------------------------------------------------
 constexpr int kTapMax = 8;
 // Coefficients per tile and band.  8 rows (halo 1.5x, 24 KB of shared memory per
@@ -363,7 +364,9 @@ __device__ __forceinline__ void cs_store(const InvArgs& f, size_t o, float2 v) {
   f.o0[o] = v;
 }
 
-// One synthesis level on tiles of 2 kFuseTY x 2 kFuseTX outputs.
+// One synthesis level on tiles of 2 kFuseTY x 2 kFuseTX outputs.  The tap of an output
+// depends on its parity, so the filters are indexed at run time: the compiler keeps
+// a copy of them in local memory (72 bytes of stack) and each tap is a load from there.
 template <int STORE>
 __global__ void __launch_bounds__(kFuseThreads) k_cs_inv(InvArgs f, Wavelet w) {
   constexpr int TX = kFuseTX, TY = kFuseTY, HB = kTapMax / 2 - 1, CY = TY + HB, CX = TX + HB;
@@ -424,6 +427,11 @@ __global__ void __launch_bounds__(kFuseThreads) k_cs_inv(InvArgs f, Wavelet w) {
 // consecutive lanes along the row, columns with consecutive lanes across them.
 // A latency-bound chain of 4 passes per level: 1024 threads, one (approximation,
 // detail) pair or one sample each and a barrier per pass.
+// kCoreSide 96 against 48 (one more level as tiled launches, the core 19 -> 7 us for
+// one 320 x 320 image): kernel time of an iteration 37 -> 33 us for one image, equal
+// for 48, 4 % more for 64 of 128 x 128 -- but two more launches, and whole calls are slower:
+// reconstruction of one 320 x 320 image 7.84 against 8.04 ms, Jacobian map of 48
+// probes 160.5 against 161.4 ms, 40 replicas at 256 x 256 equal within 0.4 %.
 constexpr int kCoreSide = 96;
 constexpr int kCoreThreads = 1024;
 

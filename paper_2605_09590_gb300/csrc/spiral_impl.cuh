@@ -306,6 +306,13 @@ __global__ void __launch_bounds__(ColsW<P1, P2>::NT, (ColsW<P1, P2>::blocks(PAD 
 // The grid rows of a step arrive by one TMA tensor load per coil, in the
 // swizzled exchange layout, and are transformed in place; those of the next
 // step are requested as soon as the a-jobs hold their last coil in registers.
+// The 128 registers of four blocks per SM do not hold z, y, the accumulators and
+// the addresses for P1 >= 20: 128 threads spill 92 bytes a thread at L = 480 padded,
+// 164 unpadded, 96 at 384 and 68 at 320 unpadded.  Three blocks of up to 168
+// registers without spills are slower all the same, except at 480 x 480 masks
+// (inside CG: 96 images of 240 x 240, 20 coils, 505 us with four blocks, 536 with three;
+// 48 of a 320 x 320 mask, 15 coils, 283 and 318; 32 of 384 x 384, 8 coils, 171 and
+// 183; 24 of 480 x 480, 8 coils, 242 and 222).
 template <int P1, int P2, bool CG, bool PAD, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT)
     k_toep_rows_inv(SpiralOp op, const __grid_constant__ CUtensorMap mG, const float2* __restrict__ xin,
