@@ -162,12 +162,12 @@ def kernel_digest(*names):
 GRAM_FILES = ("gram.cu", "tc_util.cuh", "kernels.cuh", "f16_split.cuh")
 PERSIST_FILES = ("colcg_persist.cu", "tc_util.cuh", "kernels.cuh", "f16_split.cuh")
 TRAFFIC = {
-    ("knee320_r2", 256, "gram", "1d01b2522f49a155"): (714.505728e6 + 378.052864e6 + 713.128192e6 + 375.682560e6) / 2,
-    ("knee320_r2", 256, "persist", "a0617cf5af7283d1"): (473.113856e6 + 375.561728e6 + 473.358336e6 + 373.248256e6) / 2,
+    ("knee320_r2", 256, "gram", "dae78d2d9b5c7246"): (712.295424e6 + 378.682368e6 + 712.774656e6 + 376.158208e6) / 2,
+    ("knee320_r2", 256, "persist", "2678f0e58b62aca3"): (473.599744e6 + 375.535872e6 + 473.390336e6 + 372.610816e6) / 2,
     # one spiral normal operator = k_toep_rows_fwd + k_toep_cols_w + k_toep_rows_inv (two of each averaged)
-    ("spiral240_r2", 256, "fft", "188d8e988e3ab7fe"): ((4720.863488e6 + 4658.663168e6 + 4720.915712e6 + 4655.494144e6)
-                                                       + (5021.168128e6 + 170.465792e6 + 5022.122240e6 + 170.078208e6)
-                                                       + (418.384384e6 + 4771.740160e6 + 415.642368e6 + 4772.048896e6)) / 2,
+    ("spiral240_r2", 256, "fft", "4d961a76f1cc0b92"): ((4720.321792e6 + 4658.136576e6 + 4720.184320e6 + 4655.105280e6)
+                                                       + (5016.726272e6 + 170.955776e6 + 5019.488000e6 + 170.174976e6)
+                                                       + (419.408640e6 + 4771.832576e6 + 416.948992e6 + 4772.080384e6)) / 2,
 }
 
 
