@@ -210,10 +210,9 @@ __global__ void k_axpy_bcast(float2* __restrict__ x, const float2* __restrict__ 
 // instead of one launch per direction and level and one per element-wise step:
 // 5 launches per iteration of a 4-level transform at 320 x 320 in place of
 // 19-20, the images cross memory once per level and direction instead of twice,
-// and the element-wise steps take no pass of their own (320 x 320, kernel time of
-// an iteration: 48 images 367 us as single passes, 147 us fused; one image 84 and
-// 37 us).  The arithmetic of every value is that of the
-// single passes (rows before columns in the analysis, columns before rows in the
+// and the element-wise steps take no pass of their own (320 x 320, an iteration
+// without its normal operator: 48 images 367 us as single passes, 164 us fused; one
+// image 84 and 42 us).  The arithmetic of every value is that of the single passes (rows before columns in the analysis, columns before rows in the
 // synthesis, taps in the same order).  Bound by shared memory, local memory (the
 // synthesis taps below) and the loads of the level-0 kernels for many images, by
 // the latency of each launch for one.
