@@ -212,10 +212,11 @@ __global__ void k_axpy_bcast(float2* __restrict__ x, const float2* __restrict__ 
 // 19-20, the images cross memory once per level and direction instead of twice,
 // and the element-wise steps take no pass of their own (320 x 320, an iteration
 // without its normal operator: 48 images 367 us as single passes, 164 us fused; one
-// image 84 and 42 us).  The arithmetic of every value is that of the single passes (rows before columns in the analysis, columns before rows in the
-// synthesis, taps in the same order).  Bound by shared memory, local memory (the
-// synthesis taps below) and the loads of the level-0 kernels for many images, by
-// the latency of each launch for one.
+// image 84 and 42 us).  The arithmetic of every value is that of the single passes
+// (rows before columns in the analysis, columns before rows in the synthesis, taps
+// in the same order).  Bound by shared memory, local memory (the synthesis taps
+// below) and the loads of the level-0 kernels for many images, by the latency of
+// each launch for one.
 // ---------------------------------------------------------------------------
 constexpr int kTapMax = 8;
 // Coefficients per tile and band.  8 rows (halo 1.5x, 24 KB of shared memory per
